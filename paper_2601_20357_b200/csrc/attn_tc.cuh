@@ -11,8 +11,8 @@
 //     (16 positions, resp. 16 dims, as its rows) and the query heads that share the KV head as the 8
 //     columns of B, so a tile costs half the mma it would with the (at most 8) heads as the 16 rows;
 //     the contraction is far from the tensor roofline, the point is to keep the issue slots free.
-//     q and the softmax weights are split into a bf16 head and a bf16 remainder (two products each),
-//     K and V are bf16 already, so products are exact to ~2^-17 relative and the sums are fp32;
+//     q, K and V are bf16 values already, the softmax weights are split into a bf16 head and a bf16
+//     remainder (two products), so products are exact to ~2^-17 relative and the sums are fp32;
 //   * a warp owns 16 positions of every chunk and carries its own running (max, sum, output) in
 //     registers across the chunks of a segment (the part of one cache that this CTA owns).  The
 //     warps run free of one another: each waits for a stage's "full" mbarrier on its own and
@@ -21,8 +21,10 @@
 //     the last warp to finish a segment combines the eight states and writes the result, while
 //     the others are already in the next segment.  q of a cache rides along with the first tile of its segment (one more
 //     bulk copy onto the same mbarrier);
-//   * segments of a cache that spans several CTAs are combined by the warp that finishes last
-//     (ticket), in CTA order, reading the partial results from L2;
+//   * segments of a cache that spans several CTAs are combined by the warp that finishes last (ticket), reading the
+//     partial results from L2 all at once (lane = segment for the maxima and sums).  With few chunks per CTA this tail is
+//     as long as the streaming (18 caches of 200 - 2000 positions: CTAs that combine ended 8 us after the others, now 4),
+//     so it has no 64-bit division and no load that waits for another one of its kind;
 //   * exponentials are taken in base 2 (scores pre-multiplied by log2 e, ex2.approx: relative
 //     error 2^-22).
 // Rows past a slot's position inside the last tile are masked (score -inf, weight 0); the caches are
@@ -48,6 +50,7 @@ constexpr int kAtcTile = kAtcSplit * kAtcHd * 2;   // bytes of one K (or V) tile
 constexpr int kAtcMaxStages = 8;
 constexpr int kAtcMaxCtas = 1024;
 constexpr int kAtcMaxSlots = 512;
+constexpr int kAtcMaxCap = 1 << 20;          // positions of a row that fit the packed slot table
 constexpr unsigned kAtcMaxDynSmem = 220u * 1024u;   // dynamic shared memory of a CTA that has the SM to itself (static: ~3 KB)
 
 struct AttnTcArgs {
@@ -59,7 +62,7 @@ struct AttnTcArgs {
   int* tickets;                              // [n_slots][Hkv], zero on entry and on exit
   float* out;                                // [n_slots][H][hd]; unused when act_out is given
   unsigned char* act_out;                    // or null: the output as the bf16 B operand of the next projection
-  int act_npad;                              //   (core-matrix layout of k_gemm_tc for act_npad slots, K = H * hd)
+  int act_npad, act_chunks;                  //   (tc_act_offset: tiles of act_npad slots, act_chunks blocks each; K = H * hd)
   float scale;
   int* err;
   int n_stages;
@@ -109,6 +112,7 @@ k_attn_tc_bf16(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
   __shared__ uint64_t empty[kAtcMaxStages];     // a stage's tiles have been read by all eight warps
   __shared__ int s_seg[kAtcMaxStages + 1];      // warps that have finished a segment (ring of n_stages + 1 segments)
   __shared__ int s_pref[kAtcMaxSlots + 1];
+  __shared__ unsigned s_rp[kAtcMaxSlots];       // (row << 20) | position: every slot is read from global memory once
   __shared__ int s_start;
   if (tid == 0) {
     for (int i = 0; i < n_stages; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], NW); }
@@ -117,8 +121,11 @@ k_attn_tc_bf16(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
   }
   pdl_wait();                                   // the slot table, q and the appended K, V come from the kernels before
   // chunks before every slot (prefix sums), built by the whole CTA
-  for (int i = tid; i < n_slots; i += kAtcThreads)
-    s_pref[i + 1] = slots[i].active ? Hkv * ((slots[i].pos + SPLIT) / SPLIT) : 0;
+  for (int i = tid; i < n_slots; i += kAtcThreads) {
+    const int4 sd = *reinterpret_cast<const int4*>(slots + i);                // row, pos, active
+    s_rp[i] = ((unsigned)sd.x << 20) | (unsigned)sd.y;
+    s_pref[i + 1] = sd.z ? Hkv * ((sd.y + SPLIT) / SPLIT) : 0;
+  }
   __syncthreads();
   if (warp == 0) {
     int carry = 0;
@@ -133,7 +140,13 @@ k_attn_tc_bf16(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
   }
   __syncthreads();
   const int T = s_pref[n_slots];
-  const int g_lo = (int)((long long)cta * T / NC), g_hi = (int)((long long)(cta + 1) * T / NC);
+  // contiguous ranges whose lengths differ by at most one chunk; the CTAs with chunks come first
+  const int per_cta = T / NC, extra = T - per_cta * NC;
+  const int g_lo = cta * per_cta + min(cta, extra), g_hi = g_lo + per_cta + (cta < extra ? 1 : 0);
+  auto cta_of = [&](int g) {
+    const int first = extra * (per_cta + 1);
+    return g < first ? g / (per_cta + 1) : extra + (g - first) / per_cta;
+  };
   for (int i = tid; i < n_slots; i += kAtcThreads)
     if (s_pref[i] <= g_lo && g_lo < s_pref[i + 1]) s_start = i;
   struct Walk { int s, gk, split, nsplit, row, pos; };
@@ -143,8 +156,8 @@ k_attn_tc_bf16(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
       w.split = 0; w.gk++;
       if (w.gk == Hkv) {
         w.gk = 0;
-        do { w.s++; } while (w.s < n_slots && !slots[w.s].active);
-        if (w.s < n_slots) { w.row = slots[w.s].row; w.pos = slots[w.s].pos; }
+        do { w.s++; } while (w.s < n_slots && s_pref[w.s + 1] == s_pref[w.s]);      // (inactive slots have no chunks)
+        if (w.s < n_slots) { w.row = (int)(s_rp[w.s] >> 20); w.pos = (int)(s_rp[w.s] & 0xFFFFFu); }
         w.nsplit = (w.pos + SPLIT) / SPLIT;
       }
     }
@@ -152,7 +165,7 @@ k_attn_tc_bf16(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
   auto seek = [&](int g, Walk& w) {                 // the (slot, head, split) of global chunk g < T
     int lo = 0, hi = n_slots;
     while (hi - lo > 1) { const int mid = (lo + hi) >> 1; if (s_pref[mid] <= g) lo = mid; else hi = mid; }
-    w.s = lo; w.row = slots[lo].row; w.pos = slots[lo].pos;
+    w.s = lo; w.row = (int)(s_rp[lo] >> 20); w.pos = (int)(s_rp[lo] & 0xFFFFFu);
     w.nsplit = (w.pos + SPLIT) / SPLIT;
     const int rem = g - s_pref[lo];
     w.gk = rem / w.nsplit; w.split = rem - w.gk * w.nsplit;
@@ -172,9 +185,7 @@ k_attn_tc_bf16(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
   auto store_out = [&](int s, int head, float x0, float x1) {
     if (A.act_out) {
       const int k = head * HD + 2 * lane;          // column of the projection's input
-      unsigned char* blk = A.act_out + (size_t)(k / kTcKC) * tc_block_bytes(A.act_npad);
-      *reinterpret_cast<uint32_t*>(blk + ((size_t)((k % kTcKC) >> 3) * (A.act_npad >> 3) + (s >> 3)) * 128 + (s & 7) * 16 + (k & 7) * 2) =
-          pack_bf16(x0, x1);
+      *reinterpret_cast<uint32_t*>(A.act_out + tc_act_offset(s, k, A.act_npad, A.act_chunks) + (k & 7) * 2) = pack_bf16(x0, x1);
     } else {
       *reinterpret_cast<float2*>(A.out + ((size_t)s * H + head) * HD + 2 * lane) = make_float2(x0, x1);
     }
@@ -185,7 +196,7 @@ k_attn_tc_bf16(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
   if (g_lo < g_hi) {
     const int rem = g_lo - s_pref[s_start];
     cur.s = s_start;
-    cur.row = slots[s_start].row; cur.pos = slots[s_start].pos;
+    cur.row = (int)(s_rp[s_start] >> 20); cur.pos = (int)(s_rp[s_start] & 0xFFFFFu);
     cur.nsplit = (cur.pos + SPLIT) / SPLIT;
     cur.gk = rem / cur.nsplit;
     cur.split = rem - cur.gk * cur.nsplit;
@@ -198,11 +209,11 @@ k_attn_tc_bf16(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
   // per-warp running state of the current segment.  The products are taken with the POSITIONS (scores) and the DIMS
   // (output) as the 16 rows of the A operand and the group's query heads as the 8 columns of B: a cache tile is then
   // covered by half as many mma as with the heads as rows (of which at most 8 of 16 would be used).
-  //   scores^T [16 positions x 8 heads] = K [16 x 64] q^T [64 x 8]          (4 k-steps, q as bf16 head + remainder)
+  //   scores^T [16 positions x 8 heads] = K [16 x 64] q^T [64 x 8]          (4 k-steps; q holds bf16 values)
   //   out^T    [64 dims x 8 heads]     += V^T [64 x 16] P^T [16 x 8]        (4 m-tiles, P as bf16 head + remainder)
   // Lane (g, t) holds columns (heads) 2t, 2t+1 of rows g, g+8; the softmax weights change from accumulator layout
   // (positions as rows) to B-operand layout (positions as the summed index) with movmatrix.
-  uint32_t qh[4][2], ql[4][2];                  // B fragments of q^T per k-step (column g = head g; zero beyond the group)
+  uint32_t qh[4][2];                            // B fragments of q^T per k-step (column g = head g; zero beyond the group)
   float o[4][4];                                // out^T: m-tile j = dims 16j .. 16j+15
   float m_run[2] = {-INFINITY, -INFINITY}, l_run[2] = {0.0f, 0.0f};      // heads 2t, 2t+1; maxima in base-2 units
   int seg_first_split = 0, st = 0, seg_buf = 0;
@@ -238,30 +249,29 @@ k_attn_tc_bf16(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
           a = *reinterpret_cast<const float2*>(qrow + kk * 16 + 2 * t4);
           b = *reinterpret_cast<const float2*>(qrow + kk * 16 + 8 + 2 * t4);
         }
-        split_bf16x2(a.x, a.y, qh[kk][0], ql[kk][0]);
-        split_bf16x2(b.x, b.y, qh[kk][1], ql[kk][1]);
+        qh[kk][0] = pack_bf16(a.x, a.y);
+        qh[kk][1] = pack_bf16(b.x, b.y);
       }
     }
     if (warp * 16 < cnt) {
       const uint32_t kst = smem_u32(stage0 + (size_t)st * 2 * kAtcTile), vst = kst + kAtcTile;
-      // scores of the warp's 16 positions for all heads of the group; four accumulators (q's head / remainder,
-      // even / odd k-step) keep the dependent chains two mma long
-      float sc[4][4];
+      // scores of the warp's 16 positions for all heads of the group; two accumulators (even / odd k-step) keep the
+      // dependent chains two mma long
+      float sc[2][4];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) sc[j][0] = sc[j][1] = sc[j][2] = sc[j][3] = 0.0f;
+      for (int j = 0; j < 2; ++j) sc[j][0] = sc[j][1] = sc[j][2] = sc[j][3] = 0.0f;
       const uint32_t krow = kst + (uint32_t)(warp * 16 + (ti & 1) * 8 + r8) * 128u;
 #pragma unroll
       for (int kk = 0; kk < 4; ++kk) {
         uint32_t ka[4];
         ldsm_x4(ka, krow + (uint32_t)(((2 * kk + (ti >> 1)) ^ r8) << 4));
         mma_bf16(sc[kk & 1], ka, qh[kk]);
-        mma_bf16(sc[2 + (kk & 1)], ka, ql[kk]);
       }
       // softmax over the 16 positions, base 2: entries 0, 1 belong to position g, entries 2, 3 to position g + 8
       float sv[4];
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
-        sv[e] = ((sc[0][e] + sc[1][e]) + (sc[2][e] + sc[3][e])) * scale2;
+        sv[e] = (sc[0][e] + sc[1][e]) * scale2;
         if (cnt < SPLIT && warp * 16 + (e >> 1) * 8 + g >= cnt) sv[e] = -INFINITY;
       }
       float mx0 = fmaxf(sv[0], sv[2]), mx1 = fmaxf(sv[1], sv[3]);
@@ -346,17 +356,13 @@ k_attn_tc_bf16(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
       if (last) {
         const int s = cur.s, gk = cur.gk;
         const bool whole = seg_first_split == 0 && split == nsplit - 1;
-        const int g0 = gi - split;                 // first chunk of this cache
-        int n_c = 0, c_a = 0;
+        int n_c = 0, seg = 0;                      // CTAs that the cache spans; this CTA's place among them
         if (!whole) {
-          c_a = (int)((((long long)g0 + 1) * NC - 1) / T);
-          n_c = (int)((((long long)g0 + nsplit) * NC - 1) / T) - c_a + 1;
+          const int g0 = gi - split;               // first chunk of this cache
+          const int c_a = cta_of(g0);
+          n_c = cta_of(g0 + nsplit - 1) - c_a + 1;
+          seg = cta - c_a;
         }
-        // first split of CTA (c_a + j)'s segment of this cache, or -1 when that CTA has no chunk at all
-        auto seg_of = [&](int j) {
-          const int lo_c = (int)((long long)(c_a + j) * T / NC), hi_c = (int)((long long)(c_a + j + 1) * T / NC);
-          return (lo_c < hi_c) ? max(lo_c, g0) - g0 : -1;
-        };
 #pragma unroll 1
         for (int t = 0; t < grp; ++t) {
           float M = -INFINITY;
@@ -375,7 +381,7 @@ k_attn_tc_bf16(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
           if (whole) {
             store_out(s, head, v.x / l, v.y / l);
           } else {
-            const size_t pi = ((size_t)s * H + head) * A.max_splits + seg_first_split;
+            const size_t pi = ((size_t)s * H + head) * A.max_splits + seg;
             *reinterpret_cast<float2*>(A.part_o + pi * HD + 2 * lane) = v;
             if (lane == 0) { A.part_ml[pi * 2] = M; A.part_ml[pi * 2 + 1] = l; }
           }
@@ -385,30 +391,49 @@ k_attn_tc_bf16(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
           int fin = 0;
           if (lane == 0) {
             __threadfence();                       // the warp's partial results before the ticket
-            int n_seg = 0;
-            for (int j = 0; j < n_c; ++j) n_seg += seg_of(j) >= 0;
-            fin = atomicAdd(A.tickets + s * Hkv + gk, 1) == n_seg - 1;
+            fin = atomicAdd(A.tickets + s * Hkv + gk, 1) == n_c - 1;
             if (fin) __threadfence();
           }
           fin = __shfl_sync(FULL, fin, 0);
-          if (fin) {                               // every segment of the cache is in L2: combine them in CTA order
+          if (fin) {                               // every segment of the cache is in L2: combine them
 #pragma unroll 1
             for (int t = 0; t < grp; ++t) {
               const int head = gk * grp + t;
               const size_t base = ((size_t)s * H + head) * A.max_splits;
-              float M = -INFINITY;
-              for (int j = 0; j < n_c; ++j) { const int f0 = seg_of(j); if (f0 >= 0) M = fmaxf(M, __ldcg(A.part_ml + (base + f0) * 2)); }
+              const float2* ml_p = reinterpret_cast<const float2*>(A.part_ml) + base;
+              const float2* o_p = reinterpret_cast<const float2*>(A.part_o + base * HD) + lane;
+              float2 x0[4];                        // the first four segments' outputs are requested together with the maxima
+#pragma unroll
+              for (int e = 0; e < 4; ++e) x0[e] = e < n_c ? __ldcg(o_p + (size_t)e * (HD / 2)) : make_float2(0.0f, 0.0f);
+              const float2 ml0 = lane < n_c ? __ldcg(ml_p + lane) : make_float2(-INFINITY, 0.0f);
+              float M = ml0.x;
+#pragma unroll 1
+              for (int j = 32 + lane; j < n_c; j += 32) M = fmaxf(M, __ldcg(ml_p + j).x);
+              M = warp_max_f32(M);
               float2 num = make_float2(0.0f, 0.0f);
               float den = 0.0f;
-              for (int j = 0; j < n_c; ++j) {
-                const int f0 = seg_of(j);
-                if (f0 < 0) continue;
-                const float2 ml = __ldcg(reinterpret_cast<const float2*>(A.part_ml + (base + f0) * 2));
-                const float f = ex2_approx(ml.x - M);
-                const float2 x = __ldcg(reinterpret_cast<const float2*>(A.part_o + (base + f0) * HD + 2 * lane));
-                num.x = fmaf(f, x.x, num.x); num.y = fmaf(f, x.y, num.y);
+#pragma unroll 1
+              for (int j0 = 0; j0 < n_c; j0 += 32) {
+                const float2 ml = j0 == 0 ? ml0 : (j0 + lane < n_c ? __ldcg(ml_p + j0 + lane) : make_float2(-INFINITY, 0.0f));
+                const float f = ex2_approx(ml.x - M);                       // 0 beyond the last segment
                 den = fmaf(f, ml.y, den);
+                const int cnt = min(32, n_c - j0);
+#pragma unroll 1
+                for (int j = 0; j < cnt; j += 4) {
+                  float2 x[4];
+#pragma unroll
+                  for (int e = 0; e < 4; ++e) {
+                    x[e] = x0[e];
+                    if (j0 + j > 0) x[e] = j + e < cnt ? __ldcg(o_p + (size_t)(j0 + j + e) * (HD / 2)) : make_float2(0.0f, 0.0f);
+                  }
+#pragma unroll
+                  for (int e = 0; e < 4; ++e) {
+                    const float fj = __shfl_sync(FULL, f, (j + e) & 31);
+                    num.x = fmaf(fj, x[e].x, num.x); num.y = fmaf(fj, x[e].y, num.y);
+                  }
+                }
               }
+              den = warp_sum_f32(den);
               store_out(s, head, num.x / den, num.y / den);
             }
             if (lane == 0) A.tickets[s * Hkv + gk] = 0;

@@ -68,6 +68,7 @@ struct StepArgs {
   int* last_slot;                      // [R]
   float* x;                            // [2R][d] residual stream
   int* err; int kv_capacity;
+  float* ss; int n_ss;                 // optional: partial sums of squares of the rows [slot][n_ss] (all in the first)
 };
 
 // grid: number of slots of the step; block 128
@@ -108,12 +109,19 @@ __global__ void k_begin_step(StepArgs A, const T* __restrict__ embed) {
   if (threadIdx.x == 0) A.slots[s] = SlotDesc{row, pos, active, 0};
   if (!active) return;
   float* xo = A.x + (long long)s * A.d;
+  float ss = 0.0f;
   if (src_embed) {
-    for (int i = threadIdx.x; i < A.d; i += blockDim.x) xo[i] = src_embed[i];
+    for (int i = threadIdx.x; i < A.d; i += blockDim.x) { const float v = src_embed[i]; xo[i] = v; ss = fmaf(v, v, ss); }
   } else {
     const T* e = embed + (long long)tok * A.d;
-    for (int i = threadIdx.x; i < A.d; i += blockDim.x) xo[i] = Elem<T>::load(e + i);
+    for (int i = threadIdx.x; i < A.d; i += blockDim.x) { const float v = Elem<T>::load(e + i); xo[i] = v; ss = fmaf(v, v, ss); }
   }
+  if (!A.ss) return;
+  __shared__ float red[4];
+  ss = warp_sum_f32(ss);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ss;
+  __syncthreads();
+  for (int j = threadIdx.x; j < A.n_ss; j += blockDim.x) A.ss[(size_t)s * A.n_ss + j] = j == 0 ? (red[0] + red[1]) + (red[2] + red[3]) : 0.0f;
 }
 
 // Pooled multimodal drafting input (Sec. 5, "Pooled Multimodal Drafting (P)"): visual tokens on a row-major
@@ -303,41 +311,15 @@ __global__ void __launch_bounds__(kGemvThreads) k_gemv(GemvArgs A) {
 // cache at the slot's position.  Pairs (i, i + hd/2), angle pos * theta^(-2i/hd) from a table.
 // Cache layout [R][L][Hkv][cap][hd].   grid (slots), block 128.
 // ------------------------------------------------------------------------------------------------
-// part != nullptr: the QKV projection is still ks split-K slabs [ks][slab], summed here in slab order.
-// One thread handles one rotation pair (or two v elements) at a time and requests all the slabs' values of it
-// before it adds any, so that a slot costs one or two trips to L2, not one per slab.
-constexpr int kRopeMaxSlabs = 8;
 template <typename T>
 __global__ void k_rope_append(float* __restrict__ qkv, const SlotDesc* __restrict__ slots, int H, int Hkv, int hd,
                               const float* __restrict__ rope_cos, const float* __restrict__ rope_sin,
-                              T* __restrict__ kc, T* __restrict__ vc, int layer, int L, int cap,
-                              const float* __restrict__ part = nullptr, int ks = 0, size_t slab = 0) {
-  pdl_trigger();
-  pdl_wait();
+                              T* __restrict__ kc, T* __restrict__ vc, int layer, int L, int cap) {
   const int s = blockIdx.x;
   const SlotDesc sd = slots[s];
   if (!sd.active) return;
   const int half = hd >> 1;
   float* row = qkv + (long long)s * (H + 2 * Hkv) * hd;
-  const float* prow = part ? part + (long long)s * (H + 2 * Hkv) * hd : nullptr;
-  // values of two columns, the slabs added in slab order
-  auto value2 = [&](int col_a, int col_b, float& va, float& vb) {
-    if (!prow) { va = row[col_a]; vb = row[col_b]; return; }
-    if (ks <= kRopeMaxSlabs) {
-      float a[kRopeMaxSlabs], b2[kRopeMaxSlabs];
-#pragma unroll
-      for (int k = 0; k < kRopeMaxSlabs; ++k) {
-        a[k] = k < ks ? prow[(size_t)k * slab + col_a] : 0.0f;
-        b2[k] = k < ks ? prow[(size_t)k * slab + col_b] : 0.0f;
-      }
-      va = 0.0f; vb = 0.0f;
-#pragma unroll
-      for (int k = 0; k < kRopeMaxSlabs; ++k) if (k < ks) { va += a[k]; vb += b2[k]; }
-    } else {
-      va = 0.0f; vb = 0.0f;
-      for (int k = 0; k < ks; ++k) { va += prow[(size_t)k * slab + col_a]; vb += prow[(size_t)k * slab + col_b]; }
-    }
-  };
   const float* c = rope_cos + (long long)sd.pos * half;
   const float* sn = rope_sin + (long long)sd.pos * half;
   // q heads and k heads: (H + Hkv) * half pairs
@@ -345,8 +327,7 @@ __global__ void k_rope_append(float* __restrict__ qkv, const SlotDesc* __restric
     const int head = idx / half, i = idx - head * half;
     float* p = row + head * hd;
     const float ci = c[i], si = sn[i];
-    float x1, x2;
-    value2(head * hd + i, head * hd + i + half, x1, x2);
+    const float x1 = p[i], x2 = p[i + half];
     const float r1 = x1 * ci - x2 * si;
     const float r2 = x2 * ci + x1 * si;
     if (head < H) {
@@ -360,9 +341,8 @@ __global__ void k_rope_append(float* __restrict__ qkv, const SlotDesc* __restric
   for (int idx = threadIdx.x; idx < Hkv * half; idx += blockDim.x) {
     const int g = idx / half, i = idx - g * half;
     T* dst = vc + ((((long long)sd.row * L + layer) * Hkv + g) * cap + sd.pos) * hd;
-    float v1, v2;
-    value2((H + Hkv) * hd + g * hd + i, (H + Hkv) * hd + g * hd + i + half, v1, v2);
-    Elem<T>::store(dst + i, v1); Elem<T>::store(dst + i + half, v2);
+    const float* p = row + (H + Hkv) * hd + g * hd;
+    Elem<T>::store(dst + i, p[i]); Elem<T>::store(dst + i + half, p[i + half]);
   }
 }
 
@@ -509,6 +489,8 @@ __global__ void __launch_bounds__(kAttnBwThreads, 3)
 k_attn_split_bf16(const float* __restrict__ qkv, const SlotDesc* __restrict__ slots, int H, int Hkv,
                   const __nv_bfloat16* __restrict__ kc, const __nv_bfloat16* __restrict__ vc, int layer, int L, int cap,
                   float* __restrict__ part_o, float* __restrict__ part_ml, int max_splits, float scale) {
+  pdl_trigger();
+  pdl_wait();
   constexpr int LPR = HD / 8, PPW = 32 / LPR, NW = kAttnBwThreads / 32, PPB = NW * PPW, SPLIT = kAttnBwPasses * PPB;
   const int s = blockIdx.z, g = blockIdx.y, split = blockIdx.x;
   const SlotDesc sd = slots[s];
@@ -603,11 +585,22 @@ k_attn_split_bf16(const float* __restrict__ qkv, const SlotDesc* __restrict__ sl
   }
 }
 
-// merge the splits in fixed order; grid (H, slots), block HD
+// Operand blocks of the tensor-core projections for any number of slots: slots are cut into tiles of n_pad (a multiple of
+// 16, at most 256), a tile is k_chunks blocks of 128 columns in the canonical K-major no-swizzle layout (8 rows x 16 bytes
+// core matrices).  Byte offset of the 16-byte piece that holds (slot, columns k .. k + 7).
+__host__ __device__ inline size_t tc_act_offset(int slot, int k, int n_pad, int k_chunks) {
+  const int t = slot / n_pad, r = slot - t * n_pad;
+  return ((size_t)t * k_chunks + k / 128) * ((size_t)n_pad * 256) + ((size_t)((k % 128) >> 3) * (n_pad >> 3) + (r >> 3)) * 128 + (r & 7) * 16;
+}
+
+// merge the splits in fixed order; grid (H, slots), block HD.  act_out (optional): the result goes there, rounded, as the
+// operand of the next projection, instead of into out.
 template <int HD>
 __global__ void k_attn_merge(const SlotDesc* __restrict__ slots, int H, int split_len,
                              const float* __restrict__ part_o, const float* __restrict__ part_ml, int max_splits,
-                             float* __restrict__ out) {
+                             float* __restrict__ out, unsigned char* __restrict__ act_out = nullptr, int act_npad = 0, int act_chunks = 0) {
+  pdl_trigger();
+  pdl_wait();
   const int s = blockIdx.y, head = blockIdx.x, dd = threadIdx.x;
   const SlotDesc sd = slots[s];
   if (!sd.active) return;
@@ -621,7 +614,9 @@ __global__ void k_attn_merge(const SlotDesc* __restrict__ slots, int H, int spli
     num = fmaf(f, part_o[(base + j) * HD + dd], num);
     den = fmaf(f, part_ml[(base + j) * 2 + 1], den);
   }
-  out[(long long)s * H * HD + head * HD + dd] = num / den;
+  const int k = head * HD + dd;
+  if (act_out) *reinterpret_cast<__nv_bfloat16*>(act_out + tc_act_offset(s, k, act_npad, act_chunks) + (k & 7) * 2) = __float2bfloat16_rn(num / den);
+  else out[(long long)s * H * HD + k] = num / den;
 }
 
 }  // namespace tabed

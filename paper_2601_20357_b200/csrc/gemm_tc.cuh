@@ -31,7 +31,7 @@ constexpr int kTcKC = 128;         // input columns per pipeline stage
 constexpr int kTcStages = 3;        // pipeline stages (2 when more than 128 slots share the shared memory)
 constexpr int kTcMaxStages = 8;
 constexpr int kTcThreads = 256;      // eight warps: warps w and w + 4 read the same 32 accumulator lanes, half of the columns each
-constexpr int kPrefillChunk = 256;        // positions of one row prefilled as slots of one weight pass
+constexpr int kPrefillChunk = 1024;       // positions of one row prefilled as slots of one weight pass
 constexpr int kTcMaxN = 256;       // slots per launch (MMA N is their count rounded up to 16)
 __host__ __device__ inline int tc_stages(int n_pad) { return n_pad > 128 ? 2 : kTcStages; }
 
@@ -80,7 +80,6 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_gemm_tc(const TcGemmArgs G) {
   __shared__ uint32_t s_tmem;
   __shared__ int s_bad;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  pdl_trigger();
   const int m_tile = blockIdx.x / G.ks, split = blockIdx.x - m_tile * G.ks;
   // the CTA's range of the input dimension in units of one stage (kc columns); a_bytes, b_bytes = one stage of each operand
   const int per_chunk = kTcKC / G.kc;
@@ -103,6 +102,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_gemm_tc(const TcGemmArgs G) {
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  // the next kernel may be scheduled once every CTA of this one holds its tensor memory: a successor that took the
+  // columns first would wait for this grid while this grid waits for the columns
+  pdl_trigger();
   const uint32_t tmem = s_tmem;
   const unsigned char* a_src = G.a_packed + ((size_t)m_tile * G.k_chunks + c_lo) * tc_block_bytes(kTcM);
   const unsigned char* b_src = G.b_packed + (size_t)c_lo * tc_block_bytes(G.n_pad);
@@ -249,9 +251,11 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_gemm_tc(const TcGemmArgs G) {
 // ---- operand packing ------------------------------------------------------------------------------
 // Weights [rows][K] (one or two matrices concatenated: rows0 of w0 then rows1 of w1) -> blocks
 // [m_tile][k_chunk] in the canonical layout; rows beyond rows0+rows1 and columns beyond K are zero.
+// paired: a tile holds 64 rows of w0, then the same 64 rows of w1 (gate and up, for the gated product's epilogue).
 // grid (k_chunks, m_tiles), block 256.
 __global__ void k_pack_tc(const __nv_bfloat16* __restrict__ w0, int rows0, const __nv_bfloat16* __restrict__ w1, int rows1,
-                          const __nv_bfloat16* __restrict__ w2, int rows2, int K, int k_chunks, unsigned char* __restrict__ dst) {
+                          const __nv_bfloat16* __restrict__ w2, int rows2, int K, int k_chunks, unsigned char* __restrict__ dst,
+                          int paired = 0) {
   const int kc = blockIdx.x, mt = blockIdx.y;
   unsigned char* blk = dst + ((size_t)mt * k_chunks + kc) * tc_block_bytes(kTcM);
   for (int idx = threadIdx.x; idx < kTcM * (kTcKC / 8); idx += blockDim.x) {
@@ -260,7 +264,10 @@ __global__ void k_pack_tc(const __nv_bfloat16* __restrict__ w0, int rows0, const
     const int k = kc * kTcKC + k8 * 8;
     uint4 v = make_uint4(0u, 0u, 0u, 0u);
     const __nv_bfloat16* base = nullptr;
-    if (row < rows0) base = w0;
+    if (paired) {
+      row = mt * (kTcM / 2) + (r & (kTcM / 2 - 1));
+      if (row < rows0) base = r < kTcM / 2 ? w0 : w1;
+    } else if (row < rows0) base = w0;
     else if (row < rows0 + rows1) { base = w1; row -= rows0; }
     else if (row < rows0 + rows1 + rows2) { base = w2; row -= rows0 + rows1; }
     if (base && k < K) v = *reinterpret_cast<const uint4*>(base + (size_t)row * K + k);
@@ -269,12 +276,8 @@ __global__ void k_pack_tc(const __nv_bfloat16* __restrict__ w0, int rows0, const
 }
 
 // Activations fp32 [n][K] (row stride `stride`) -> bf16 blocks [k_chunk] of n_pad rows in the canonical
-// layout; optional per-row scale (RMSNorm) and bf16 gain.  Rows >= n and columns >= K are zero.
-// grid (k_chunks), block 256.
-__global__ void k_prep_act(const float* __restrict__ x, int stride, int n, int n_pad, int K, const float* __restrict__ row_scale,
-                           const __nv_bfloat16* __restrict__ gain, unsigned char* __restrict__ dst) {
-  pdl_trigger();
-  pdl_wait();
+// layout.  Rows >= n and columns >= K are zero.  grid (k_chunks), block 256.
+__global__ void k_prep_act(const float* __restrict__ x, int stride, int n, int n_pad, int K, unsigned char* __restrict__ dst) {
   const int kc = blockIdx.x;
   unsigned char* blk = dst + (size_t)kc * tc_block_bytes(n_pad);
   for (int idx = threadIdx.x; idx < n_pad * (kTcKC / 8); idx += blockDim.x) {
@@ -284,148 +287,10 @@ __global__ void k_prep_act(const float* __restrict__ x, int stride, int n, int n
     if (r < n && k < K) {
       const float4 a = *reinterpret_cast<const float4*>(x + (size_t)r * stride + k);
       const float4 b = *reinterpret_cast<const float4*>(x + (size_t)r * stride + k + 4);
-      float f[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-      if (row_scale) {
-        const float sc = row_scale[r];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) f[j] = f[j] * sc * __bfloat162float(gain[k + j]);
-      }
-      v.x = pack_bf16(f[0], f[1]); v.y = pack_bf16(f[2], f[3]); v.z = pack_bf16(f[4], f[5]); v.w = pack_bf16(f[6], f[7]);
+      v.x = pack_bf16(a.x, a.y); v.y = pack_bf16(a.z, a.w); v.z = pack_bf16(b.x, b.y); v.w = pack_bf16(b.z, b.w);
     }
     *reinterpret_cast<uint4*>(blk + ((size_t)k8 * (n_pad / 8) + (r >> 3)) * 128 + (r & 7) * 16) = v;
   }
-}
-
-// ---- activation preparation for the tensor-core projections ------------------------------------------
-// One CTA per slot of the group: x <- base + sum of the previous projection's k-split partials (written
-// back when `write_back`), optional RMSNorm (gain != null), bf16 rounding, canonical operand layout.
-// src_slot (optional) maps the group's row to the slot whose residual it reads (LM head: last slot of a row).
-struct PrepRowArgs {
-  float* x; int d;                       // residual stream [slot][d]
-  const float* partial; int ks; size_t slab;     // [ks] slabs [slot][d] or null
-  const int* src_slot;                   // or null
-  const SlotDesc* slots;                 // activity of the slots (null: all active)
-  const __nv_bfloat16* gain; float eps;  // RMSNorm gain or null
-  int slot0, n, n_pad, write_back;
-  unsigned char* dst;                    // [k_chunks] blocks of n_pad rows
-};
-__global__ void __launch_bounds__(256) k_prep_row(const PrepRowArgs P) {
-  pdl_trigger();
-  pdl_wait();
-  const int r = blockIdx.x, tid = threadIdx.x;
-  const int s = P.src_slot ? P.src_slot[P.slot0 + r] : P.slot0 + r;
-  if (P.slots && !P.slots[s].active) return;
-  __shared__ float red[8];
-  __shared__ float s_scale;
-  float* xr = P.x + (size_t)s * P.d;
-  // resolve 8 consecutive elements: the residual plus the slabs, all requested before any is added (slab order kept)
-  auto resolve = [&](int k, float (&f)[8]) {
-    const float4 a = *reinterpret_cast<const float4*>(xr + k), b = *reinterpret_cast<const float4*>(xr + k + 4);
-    f[0] = a.x; f[1] = a.y; f[2] = a.z; f[3] = a.w; f[4] = b.x; f[5] = b.y; f[6] = b.z; f[7] = b.w;
-    for (int q0 = 0; q0 < P.ks; q0 += 8) {
-      float4 c[8], e[8];
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const bool ok = q0 + j < P.ks;
-        const float* pp = P.partial + (size_t)(ok ? q0 + j : 0) * P.slab + (size_t)s * P.d + k;
-        c[j] = ok ? *reinterpret_cast<const float4*>(pp) : make_float4(0.f, 0.f, 0.f, 0.f);
-        e[j] = ok ? *reinterpret_cast<const float4*>(pp + 4) : make_float4(0.f, 0.f, 0.f, 0.f);
-      }
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        if (q0 + j < P.ks) {
-          f[0] += c[j].x; f[1] += c[j].y; f[2] += c[j].z; f[3] += c[j].w; f[4] += e[j].x; f[5] += e[j].y; f[6] += e[j].z; f[7] += e[j].w;
-        }
-      }
-    }
-  };
-  auto emit = [&](int k, const float (&f)[8], float sc) {
-    float g[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) g[j] = P.gain ? f[j] * sc * __bfloat162float(P.gain[k + j]) : f[j];
-    uint4 v;
-    v.x = pack_bf16(g[0], g[1]); v.y = pack_bf16(g[2], g[3]); v.z = pack_bf16(g[4], g[5]); v.w = pack_bf16(g[6], g[7]);
-    const int kc = k / kTcKC, k8 = (k % kTcKC) >> 3;
-    *reinterpret_cast<uint4*>(P.dst + (size_t)kc * tc_block_bytes(P.n_pad) + ((size_t)k8 * (P.n_pad / 8) + (r >> 3)) * 128 + (r & 7) * 16) = v;
-  };
-  const bool one_pass = P.d <= 256 * 8;              // every thread owns at most one group of 8: it stays in registers
-  float keep[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-  float ss = 0.0f;
-  // pass 1: resolve, write back, sum of squares.  Thread owns groups of 8 consecutive elements.
-  for (int k = tid * 8; k < P.d; k += 256 * 8) {
-    float f[8];
-    resolve(k, f);
-    if (P.write_back && P.ks > 0) {
-      *reinterpret_cast<float4*>(xr + k) = make_float4(f[0], f[1], f[2], f[3]);
-      *reinterpret_cast<float4*>(xr + k + 4) = make_float4(f[4], f[5], f[6], f[7]);
-    }
-#pragma unroll
-    for (int j = 0; j < 8; ++j) { ss = fmaf(f[j], f[j], ss); keep[j] = f[j]; }
-  }
-  ss = warp_sum_f32(ss);
-  if ((tid & 31) == 0) red[tid >> 5] = ss;
-  __syncthreads();
-  if (tid == 0) {
-    float tot = 0.0f;
-    for (int w = 0; w < 8; ++w) tot += red[w];
-    s_scale = P.gain ? 1.0f / sqrtf(tot / (float)P.d + P.eps) : 1.0f;
-  }
-  __syncthreads();
-  const float sc = s_scale;
-  // pass 2: scale, round, store 16-byte pieces of the canonical layout (long rows: resolved again, the values are in L1/L2)
-  if (one_pass) {
-    if (tid * 8 < P.d) emit(tid * 8, keep, sc);
-  } else {
-    for (int k = tid * 8; k < P.d; k += 256 * 8) {
-      float f[8];
-      if (P.write_back && P.ks > 0) {
-        const float4 a = *reinterpret_cast<const float4*>(xr + k), b = *reinterpret_cast<const float4*>(xr + k + 4);
-        f[0] = a.x; f[1] = a.y; f[2] = a.z; f[3] = a.w; f[4] = b.x; f[5] = b.y; f[6] = b.z; f[7] = b.w;
-      } else {
-        resolve(k, f);
-      }
-      emit(k, f, sc);
-    }
-  }
-}
-
-// Gated product for the down projection from the gate|up projection's partials:
-// mid[s][f] = SiLU(sum_q pg[q][s][f]) * (sum_q pg[q][s][F + f]), rounded to bf16, canonical layout.
-// grid (k_chunks of F, slots of the group), block 16 (one thread per 8 columns of the chunk).
-__global__ void k_swiglu_prep(const float* __restrict__ partial, int ks, size_t slab, int F, const SlotDesc* __restrict__ slots,
-                              int slot0, int n_pad, unsigned char* __restrict__ dst) {
-  pdl_trigger();
-  pdl_wait();
-  const int kc = blockIdx.x, r = blockIdx.y, k8 = threadIdx.x;
-  const int s = slot0 + r;
-  if (slots && !slots[s].active) return;
-  const int f0 = kc * kTcKC + k8 * 8;
-  uint4 v = make_uint4(0u, 0u, 0u, 0u);
-  if (f0 < F) {
-    float g[8] = {0, 0, 0, 0, 0, 0, 0, 0}, u[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    for (int q0 = 0; q0 < ks; q0 += 4) {              // four slabs requested together, added in slab order
-      float4 a[4], b[4], c[4], e[4];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const bool ok = q0 + j < ks;
-        const float* pg = partial + (size_t)(ok ? q0 + j : 0) * slab + (size_t)s * (2 * F) + f0;
-        const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
-        a[j] = ok ? *reinterpret_cast<const float4*>(pg) : z; b[j] = ok ? *reinterpret_cast<const float4*>(pg + 4) : z;
-        c[j] = ok ? *reinterpret_cast<const float4*>(pg + F) : z; e[j] = ok ? *reinterpret_cast<const float4*>(pg + F + 4) : z;
-      }
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        if (q0 + j >= ks) continue;
-        g[0] += a[j].x; g[1] += a[j].y; g[2] += a[j].z; g[3] += a[j].w; g[4] += b[j].x; g[5] += b[j].y; g[6] += b[j].z; g[7] += b[j].w;
-        u[0] += c[j].x; u[1] += c[j].y; u[2] += c[j].z; u[3] += c[j].w; u[4] += e[j].x; u[5] += e[j].y; u[6] += e[j].z; u[7] += e[j].w;
-      }
-    }
-    float m[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) m[j] = g[j] / (1.0f + expf(-g[j])) * u[j];
-    v.x = pack_bf16(m[0], m[1]); v.y = pack_bf16(m[2], m[3]); v.z = pack_bf16(m[4], m[5]); v.w = pack_bf16(m[6], m[7]);
-  }
-  *reinterpret_cast<uint4*>(dst + (size_t)kc * tc_block_bytes(n_pad) + ((size_t)k8 * (n_pad / 8) + (r >> 3)) * 128 + (r & 7) * 16) = v;
 }
 
 }  // namespace tabed

@@ -19,7 +19,9 @@
 #include "decide_kernels.cuh"
 #include "round_kernel.cuh"
 #include "gemm_tc.cuh"
+#include "proj_tc.cuh"
 #include "attn_tc.cuh"
+#include "prompt_attn.cuh"
 #include "request_kernels.cuh"
 
 using namespace tabed;
@@ -40,6 +42,9 @@ struct DeviceGuard {
 };
 
 }  // namespace
+
+// A layer projection's cut into slot tiles and K splits (plan_proj).
+struct ProjPlan { int n_pad, n_tiles, ks, cps, n_stages; bool norm; unsigned recv_off; size_t smem; float us; };
 
 struct tabed_handle {
   tabed_config cfg;
@@ -107,13 +112,17 @@ struct tabed_handle {
   bool tc_ok = false;                        // tcgen05 projections are set up (prefill in chunks; drafting when tc_auto)
   bool tc_auto = false;                      // ... and are the automatic choice for drafting (no persistent kernel)
   int slot_cap = 0;                          // slots the step buffers hold: 2R, or a prefill chunk if that is more
-  struct TcKind { int rows, K, m_tiles, k_chunks, ks, cps; size_t bytes; };
-  TcKind tck[5]{};                  // KIND_QKV, KIND_O, KIND_GU (gate|up rows), KIND_DN, KIND_LM
+  struct TcKind { int rows, K, m_tiles, k_chunks; size_t bytes; };
+  TcKind tck[5]{};                  // KIND_QKV, KIND_O, KIND_GU (tiles of 64 gate + 64 up rows), KIND_DN, KIND_LM
   unsigned char* tc_w = nullptr;    // [L][QKV | O | GU | DN] then LM, operand blocks of k_pack_tc
   size_t tc_layer_stride = 0, tc_off[5]{};
-  unsigned char* tc_act = nullptr;  // activation operand blocks of the group being projected
-  float *tc_pq = nullptr, *tc_po = nullptr, *tc_pgu = nullptr, *tc_pd = nullptr;   // k-split partials [ks][2R][rows]
+  unsigned char *tc_act = nullptr, *tc_mid = nullptr;   // operand blocks: normalised rows or attention outputs; gated products
+  float *tc_ss_a = nullptr, *tc_ss_m = nullptr;         // partial sums of squares of the residual [slot][n_ss], entering a
+                                                        // layer and between its attention and its MLP
   size_t tc_smem = 0;
+  struct StepPlan { int n_slots; ProjPlan p[4]; };
+  std::vector<StepPlan> step_plans;
+  int proj_fit[9]{};                // resident clusters of 1 .. 8 CTAs of a projection, one CTA per SM
   // per-kernel-class timing (tabed_profile_begin / tabed_profile_end)
   int prof_class = -1;
   std::vector<cudaEvent_t> prof_events;     // start/stop pairs
@@ -262,10 +271,10 @@ void launch_gemv(tabed_handle* h, const GemvArgs& a, int epi, int ns) {
   else { if (f32) launch_gemv_ns<float, EPI_SWIGLU>(h, a, ns); else launch_gemv_ns<__nv_bfloat16, EPI_SWIGLU>(h, a, ns); }
 }
 
-// act_out != null (and *wrote_act given): the caller wants the output as the next projection's bf16 operand blocks;
-// the kernel that can do that sets *wrote_act, otherwise the fp32 rows in h->attn_out are the result.
+// act_out != null: the output goes there as the next projection's bf16 operand blocks (tc_act_offset), otherwise as fp32
+// rows into h->attn_out.
 template <typename T, int HD>
-void launch_attention_hd(tabed_handle* h, int layer, int n_slots, int max_pos, unsigned char* act_out, int act_npad, bool* wrote_act) {
+void launch_attention_hd(tabed_handle* h, int layer, int n_slots, int max_pos, unsigned char* act_out, int act_npad, int act_chunks) {
   if constexpr (std::is_same<T, __nv_bfloat16>::value) {
     // bandwidth-oriented kernel: all K, V loads of a split in flight at once
     const int split_len = attn_bw_split_len(HD);
@@ -294,20 +303,20 @@ void launch_attention_hd(tabed_handle* h, int layer, int n_slots, int max_pos, u
           AttnTcArgs a;
           a.qkv = h->qkv; a.slots = h->slots; a.n_slots = n_slots; a.H = h->H; a.Hkv = h->Hkv; a.layer = layer; a.L = h->L;
           a.cap = h->cap; a.qkv_w = h->qkv_w; a.part_o = h->part_o; a.part_ml = h->part_ml; a.max_splits = h->max_splits;
-          a.act_out = act_out; a.act_npad = act_npad;
+          a.act_out = act_out; a.act_npad = act_npad; a.act_chunks = act_chunks;
           a.tickets = h->attn_tickets; a.out = h->attn_out; a.scale = 1.0f / sqrtf((float)h->hd); a.err = h->err; a.n_stages = n_stages;
           TABED_LAUNCH_PDL(h, k_attn_tc_bf16, n_ctas, kAtcThreads, smem2, h->tm_k, h->tm_v, a);
-          if (wrote_act) *wrote_act = act_out != nullptr;
           return;
         }
       }
     }
     if (smem <= 96 * 1024) {
-      TABED_LAUNCH(h, part, dim3(splits, h->Hkv, n_slots), kAttnBwThreads, smem, h->qkv, h->slots, h->H, h->Hkv,
+      TABED_LAUNCH_PDL(h, part, dim3(splits, h->Hkv, n_slots), kAttnBwThreads, smem, h->qkv, h->slots, h->H, h->Hkv,
                    reinterpret_cast<const __nv_bfloat16*>(h->kc), reinterpret_cast<const __nv_bfloat16*>(h->vc), layer, h->L, h->cap,
                    h->part_o, h->part_ml, h->max_splits, 1.0f / sqrtf((float)h->hd));
       auto merge = k_attn_merge<HD>;
-      TABED_LAUNCH(h, merge, dim3(h->H, n_slots), HD, 0, h->slots, h->H, split_len, h->part_o, h->part_ml, h->max_splits, h->attn_out);
+      TABED_LAUNCH_PDL(h, merge, dim3(h->H, n_slots), HD, 0, h->slots, h->H, split_len, h->part_o, h->part_ml, h->max_splits, h->attn_out,
+                       act_out, act_npad, act_chunks);
       return;
     }
   }
@@ -320,17 +329,15 @@ void launch_attention_hd(tabed_handle* h, int layer, int n_slots, int max_pos, u
                reinterpret_cast<const T*>(h->kc), reinterpret_cast<const T*>(h->vc), layer, h->L, h->cap, split_len,
                h->part_o, h->part_ml, h->max_splits, scale);
   TABED_LAUNCH(h, merge, dim3(h->H, n_slots), HD, 0, h->slots, h->H, split_len, h->part_o, h->part_ml,
-               h->max_splits, h->attn_out);
+               h->max_splits, h->attn_out, act_out, act_npad, act_chunks);
 }
 
 template <typename T>
-void launch_attention_t(tabed_handle* h, int layer, int n_slots, int max_pos, unsigned char* act_out = nullptr, int act_npad = 0,
-                        bool* wrote_act = nullptr) {
-  if (wrote_act) *wrote_act = false;
+void launch_attention_t(tabed_handle* h, int layer, int n_slots, int max_pos, unsigned char* act_out = nullptr, int act_npad = 0, int act_chunks = 0) {
   switch (h->hd) {
-    case 32: launch_attention_hd<T, 32>(h, layer, n_slots, max_pos, act_out, act_npad, wrote_act); break;
-    case 64: launch_attention_hd<T, 64>(h, layer, n_slots, max_pos, act_out, act_npad, wrote_act); break;
-    default: launch_attention_hd<T, 128>(h, layer, n_slots, max_pos, act_out, act_npad, wrote_act); break;
+    case 32: launch_attention_hd<T, 32>(h, layer, n_slots, max_pos, act_out, act_npad, act_chunks); break;
+    case 64: launch_attention_hd<T, 64>(h, layer, n_slots, max_pos, act_out, act_npad, act_chunks); break;
+    default: launch_attention_hd<T, 128>(h, layer, n_slots, max_pos, act_out, act_npad, act_chunks); break;
   }
 }
 
@@ -574,6 +581,15 @@ int launch_persistent_round(tabed_handle* h, const float* u_draft, int32_t* out_
 }
 
 // ---- tensor-core path for many rows -----------------------------------------------------------------
+// rows per tile of the LM head: all of them up to 256 (one MMA), else equal tiles
+int tc_n_pad(int n) {
+  const int tiles = (n + kTcMaxN - 1) / kTcMaxN;
+  return ((n + tiles - 1) / tiles + 15) / 16 * 16;
+}
+
+// partial sums of squares per residual row: one per 128-row tile, a multiple of 4 (the rest stay zero)
+int proj_n_ss(const tabed_handle* h) { return (h->tck[KIND_O].m_tiles + 3) & ~3; }
+
 int setup_tc(tabed_handle* h) {
   const tabed_config& c = h->cfg;
   h->tc_ok = false;
@@ -581,19 +597,16 @@ int setup_tc(tabed_handle* h) {
   cudaDeviceProp prop;
   if (cudaGetDeviceProperties(&prop, c.device) != cudaSuccess) return TABED_ERR_CUDA;
   if (prop.major < 10) return TABED_OK;
-  const int n_sm = prop.multiProcessorCount, kvd = h->Hkv * h->hd;
+  const int kvd = h->Hkv * h->hd;
   const int rows[5] = {h->qkv_w, h->d, 2 * h->F, h->d, h->V};
   const int Ks[5] = {h->d, h->H * h->hd, h->d, h->F, h->d};
   for (int k = 0; k < 5; ++k) {
     tabed_handle::TcKind& t = h->tck[k];
     t.rows = rows[k]; t.K = Ks[k];
     t.m_tiles = (t.rows + kTcM - 1) / kTcM; t.k_chunks = (t.K + kTcKC - 1) / kTcKC;
-    int ks = std::max(1, std::min(std::min(t.k_chunks, 8), (n_sm + t.m_tiles - 1) / t.m_tiles));   // at most 8 slabs to sum
-    if (k == KIND_LM) ks = 1;                       // logits are stored directly
-    t.cps = (t.k_chunks + ks - 1) / ks;
-    t.ks = (t.k_chunks + t.cps - 1) / t.cps;
-    t.bytes = (size_t)t.m_tiles * t.k_chunks * tc_block_bytes(kTcM);
   }
+  h->tck[KIND_GU].m_tiles = 2 * h->tck[KIND_DN].k_chunks;      // every column of the down projection's operand is written
+  for (int k = 0; k < 5; ++k) h->tck[k].bytes = (size_t)h->tck[k].m_tiles * h->tck[k].k_chunks * tc_block_bytes(kTcM);
   h->tc_off[KIND_QKV] = 0;
   h->tc_off[KIND_O] = h->tck[KIND_QKV].bytes;
   h->tc_off[KIND_GU] = h->tc_off[KIND_O] + h->tck[KIND_O].bytes;
@@ -604,17 +617,32 @@ int setup_tc(tabed_handle* h) {
   h->tc_smem = 0;
   for (int np = 16; np <= n_pad_max; np += 16)
     h->tc_smem = std::max(h->tc_smem, (size_t)tc_stages(np) * (tc_block_bytes(kTcM) + tc_block_bytes(np)) + 1024);
-  if (h->tc_smem > (size_t)prop.sharedMemPerBlockOptin) return TABED_OK;
-  if (cudaFuncSetAttribute(k_gemm_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)h->tc_smem) != cudaSuccess) return TABED_ERR_CUDA;
+  if (std::max(h->tc_smem, kProjMaxSmem) > (size_t)prop.sharedMemPerBlockOptin) return TABED_OK;
+  auto smem_attr = [](auto kern, size_t bytes) { return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess; };
+  if (!smem_attr(k_gemm_tc, h->tc_smem) || !smem_attr(k_proj_tc<PROJ_QKV>, kProjMaxSmem) || !smem_attr(k_proj_tc<PROJ_RESID>, kProjMaxSmem) ||
+      !smem_attr(k_proj_tc<PROJ_SWIGLU>, kProjMaxSmem) || !smem_attr(k_prompt_attn<32>, prompt_attn_smem(32)) ||
+      !smem_attr(k_prompt_attn<64>, prompt_attn_smem(64)) || !smem_attr(k_prompt_attn<128>, prompt_attn_smem(128)))
+    return TABED_ERR_CUDA;
+  // Clusters of a projection that the device keeps resident at once (an SM group does not divide evenly into every size: 148
+  // SMs hold 74 pairs but 45 threes).  The occupancy calculator gives every kernel with tensor memory the SM to itself; with
+  // half of the shared memory and of the registers two CTAs do run side by side.
+  for (int ks = 1; ks <= kProjMaxSplit; ++ks) {
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3((unsigned)ks); lc.blockDim = dim3(kTcThreads); lc.dynamicSmemBytes = kProjMaxSmem;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)ks; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    lc.attrs = at; lc.numAttrs = 1;
+    if (cudaOccupancyMaxActiveClusters(&h->proj_fit[ks], k_proj_tc<PROJ_QKV>, &lc) != cudaSuccess) return TABED_ERR_CUDA;
+  }
   int rc = TABED_OK;
-  auto A2 = [&](auto** ptr, size_t count) { if (rc == TABED_OK) rc = dev_alloc(h, ptr, count, false); };
-  const size_t S2 = (size_t)h->slot_cap;
-  int kc_max = 0;
-  for (int k = 0; k < 5; ++k) kc_max = std::max(kc_max, h->tck[k].k_chunks);
-  A2(&h->tc_w, h->tc_off[KIND_LM] + h->tck[KIND_LM].bytes);
-  A2(&h->tc_act, (size_t)kc_max * tc_block_bytes(n_pad_max));
-  A2(&h->tc_pq, (size_t)h->tck[KIND_QKV].ks * S2 * h->qkv_w); A2(&h->tc_po, (size_t)h->tck[KIND_O].ks * S2 * h->d);
-  A2(&h->tc_pgu, (size_t)h->tck[KIND_GU].ks * S2 * 2 * h->F); A2(&h->tc_pd, (size_t)h->tck[KIND_DN].ks * S2 * h->d);
+  auto A2 = [&](auto** ptr, size_t count, bool zero) { if (rc == TABED_OK) rc = dev_alloc(h, ptr, count, zero); };
+  const size_t S2 = (size_t)h->slot_cap * 3 / 2 + kTcMaxN, n_ss = proj_n_ss(h);       // (tiles of at least 32 slots, padded to 16)
+  A2(&h->tc_w, h->tc_off[KIND_LM] + h->tck[KIND_LM].bytes, false);
+  // (zeroed: columns beyond the operand's K and slots nobody wrote only meet zero weights or unused outputs, but must be finite)
+  A2(&h->tc_act, S2 * std::max(h->tck[KIND_QKV].k_chunks, h->tck[KIND_O].k_chunks) * kTcKC * 2, true);
+  A2(&h->tc_mid, S2 * h->tck[KIND_DN].k_chunks * kTcKC * 2, true);
+  A2(&h->tc_ss_a, n_ss * h->slot_cap, true); A2(&h->tc_ss_m, n_ss * h->slot_cap, true);
   if (rc != TABED_OK) return rc;
   using bf = __nv_bfloat16;
   for (int l = 0; l <= h->L; ++l) {
@@ -625,7 +653,7 @@ int setup_tc(tabed_handle* h) {
       const dim3 grid(t.k_chunks, t.m_tiles);
       if (k == KIND_QKV) k_pack_tc<<<grid, 256, 0, h->stream>>>((const bf*)h->wq[l], h->d, (const bf*)h->wk[l], kvd, (const bf*)h->wv[l], kvd, t.K, t.k_chunks, dst);
       else if (k == KIND_O) k_pack_tc<<<grid, 256, 0, h->stream>>>((const bf*)h->wo[l], h->d, nullptr, 0, nullptr, 0, t.K, t.k_chunks, dst);
-      else if (k == KIND_GU) k_pack_tc<<<grid, 256, 0, h->stream>>>((const bf*)h->w_gate[l], h->F, (const bf*)h->w_up[l], h->F, nullptr, 0, t.K, t.k_chunks, dst);
+      else if (k == KIND_GU) k_pack_tc<<<grid, 256, 0, h->stream>>>((const bf*)h->w_gate[l], h->F, (const bf*)h->w_up[l], h->F, nullptr, 0, t.K, t.k_chunks, dst, 1);
       else if (k == KIND_DN) k_pack_tc<<<grid, 256, 0, h->stream>>>((const bf*)h->w_down[l], h->d, nullptr, 0, nullptr, 0, t.K, t.k_chunks, dst);
       else k_pack_tc<<<grid, 256, 0, h->stream>>>((const bf*)h->lm_head, h->V, nullptr, 0, nullptr, 0, t.K, t.k_chunks, dst);
     }
@@ -636,95 +664,183 @@ int setup_tc(tabed_handle* h) {
   return TABED_OK;
 }
 
-// one tensor-core projection of a slot group whose operand blocks are already in h->tc_act
-void launch_gemm_tc(tabed_handle* h, int kind, int layer, int n, float* partial, size_t slab, const SlotDesc* slots, int rows_valid) {
-  const tabed_handle::TcKind& t = h->tck[kind];
+// the LM head over one tile of n rows whose operand blocks are at `act`: logits are stored directly
+void launch_lm_head_tc(tabed_handle* h, const unsigned char* act, int n, int n_pad, float* logits) {
+  const tabed_handle::TcKind& t = h->tck[KIND_LM];
   TcGemmArgs G{};
-  G.a_packed = h->tc_w + h->tc_off[kind] + (kind == KIND_LM ? 0 : (size_t)layer * h->tc_layer_stride);
-  G.b_packed = h->tc_act; G.partial = partial; G.slab = slab; G.slots = slots;
-  G.rows_total = t.rows; G.rows_valid = rows_valid; G.n_pad = (n + 15) / 16 * 16; G.n_slots = n;
-  G.k_chunks = t.k_chunks; G.ks = t.ks; G.cps = t.cps; G.err = h->err;
-  G.kc = kTcKC; G.n_stages = tc_stages(G.n_pad);
-  // More tiles than SMs (the LM head): stages of half a block, so that two CTAs share an SM and one's epilogue
-  // overlaps the other's copies (32000 x 768 for 96 slots: 28.8 -> 23.3 us); the projections with at most one CTA
-  // per SM are no faster with half stages (measured with 3, 4 and 6 of them).
-  if (t.m_tiles * t.ks > h->n_sm && G.n_pad <= 128) { G.kc = kTcKC / 2; G.n_stages = 3; }
+  G.a_packed = h->tc_w + h->tc_off[KIND_LM]; G.b_packed = act; G.partial = logits;
+  G.rows_total = t.rows; G.rows_valid = h->V; G.n_pad = n_pad; G.n_slots = n;
+  G.k_chunks = t.k_chunks; G.ks = 1; G.cps = t.k_chunks; G.err = h->err;
+  G.kc = kTcKC; G.n_stages = tc_stages(n_pad);
+  // More tiles than SMs: stages of half a block, so that two CTAs share an SM and one's epilogue overlaps the other's
+  // copies (32000 x 768 for 96 slots: 28.8 -> 23.3 us)
+  if (t.m_tiles > h->n_sm && G.n_pad <= 128) { G.kc = kTcKC / 2; G.n_stages = 3; }
   const size_t smem = (size_t)G.n_stages * (tc_block_bytes(kTcM) + tc_block_bytes(G.n_pad)) / (kTcKC / G.kc) + 1024;
-  TABED_LAUNCH_PDL(h, k_gemm_tc, t.m_tiles * t.ks, kTcThreads, smem, G);
+  TABED_LAUNCH_PDL(h, k_gemm_tc, t.m_tiles, kTcThreads, smem, G);
 }
 
-// One shared-weight decoder step over `n_slots` slots with the projections on the tensor cores.
+// How a layer projection over n_slots slots is cut into slot tiles and K splits.  What a choice costs, in us, as measured on
+// the kernel's own time line (18 - 1024 slots, 768 - 4864 columns): a CTA draws 75 KB/us alone and all of them together
+// 6.5 MB/us from L2; 8 slots of the epilogue cost each warp 0.2 us; the exchange between the CTAs of a cluster 1 us, and
+// 0.02 us per slot more where the slabs are pulled for lack of a receive buffer; a normalising prologue 1.2 us and 0.02 us per
+// slot and 128 columns, against 3 us for a launch that packs the operand; a wave that is not full costs a wave.
+ProjPlan plan_proj(const tabed_handle* h, int kind, int n_slots, bool can_norm) {
+  const tabed_handle::TcKind& t = h->tck[kind];
+  ProjPlan best{};
+  best.us = 1e30f;
+  int last_pad = 0;
+  for (int tiles = (n_slots + kTcMaxN - 1) / kTcMaxN; tiles <= std::max(1, n_slots / 32); ++tiles) {
+    const int n_pad = ((n_slots + tiles - 1) / tiles + 15) / 16 * 16;
+    if (n_pad == last_pad) continue;
+    last_pad = n_pad;
+    const int n_tiles = (n_slots + n_pad - 1) / n_pad, units = t.m_tiles * n_tiles;
+    const size_t a = tc_block_bytes(kTcM), b = tc_block_bytes(n_pad), bn = proj_norm_block_bytes(n_pad), slab = (size_t)n_pad * kTcM * sizeof(float);
+    for (int want = 1; want <= std::min(kProjMaxSplit, t.k_chunks); ++want) {
+      const int cps = (t.k_chunks + want - 1) / want, ks = (t.k_chunks + cps - 1) / cps;
+      if (ks != want) continue;
+      const size_t recv = ks > 1 ? (size_t)ks * proj_owned(n_pad, ks) * kTcM * sizeof(float) : 0;
+      const int deep = std::min(cps, kProjMaxStages), least = std::min(2, deep);
+      for (int norm = 0; norm <= (can_norm ? 1 : 0); ++norm) {
+        const size_t fixed = norm ? (size_t)cps * bn : 0, per_stage = norm ? a : a + b;
+        for (int half = 0; half < 2; ++half) {
+          const size_t budget = half ? kProjHalfSmem : kProjMaxSmem;
+          // slabs are pushed where the receive buffer fits beside the operands, else pulled
+          const size_t extra = recv && fixed + recv + least * per_stage <= budget ? recv : 0;
+          if (std::max(fixed + extra + least * per_stage, extra ? 0 : slab) > budget) continue;
+          ProjPlan p{};
+          p.n_pad = n_pad; p.n_tiles = n_tiles; p.ks = ks; p.cps = cps; p.norm = norm != 0;
+          p.n_stages = (int)std::min<size_t>(deep, (budget - fixed - extra) / per_stage);
+          const size_t operands = fixed + p.n_stages * per_stage;
+          p.recv_off = extra ? (unsigned)operands : 0u;
+          p.smem = std::max(operands + extra, extra ? 0 : slab);
+          const int fit = std::max(1, h->proj_fit[ks] * (p.smem <= kProjHalfSmem ? 2 : 1)) * ks, ctas = units * ks;
+          const float waves = (float)((ctas + fit - 1) / fit);
+          const float rate = std::min(p.n_stages >= std::min(deep, 3) ? 75.0f : 60.0f, 6500.0f / (float)std::min(ctas, fit));       // KB per us and CTA
+          p.us = waves * ((float)(cps * (a + b)) / 1024.0f / rate + 2.0f + 0.25f * (float)((proj_owned(n_pad, ks) + 7) / 8) + (ks > 1 ? 1.0f : 0.0f) +
+                          (ks > 1 && !extra ? 0.02f * (float)n_pad : 0.0f) + (norm ? 1.2f + 0.02f * (float)(std::min(n_pad, n_slots) * cps) : 0.0f)) +
+                 (can_norm && !norm ? 3.0f : 0.0f) - (p.smem <= kProjHalfSmem ? 0.5f : 0.0f);      // (room for the next kernel's start)
+          if (p.us < best.us) best = p;
+        }
+      }
+    }
+  }
+  return best;                                                 // (256 slots in one CTA: two stages are 192 KB - always found)
+}
+
+// The plans of a step, kept for the few slot counts that a handle's steps have in turn (2 R and R; a prompt's chunks).
+const tabed_handle::StepPlan& step_plan(tabed_handle* h, int n_slots) {
+  for (const auto& e : h->step_plans) if (e.n_slots == n_slots) return e;
+  tabed_handle::StepPlan e;
+  e.n_slots = n_slots;
+  e.p[KIND_QKV] = plan_proj(h, KIND_QKV, n_slots, true);
+  e.p[KIND_O] = plan_proj(h, KIND_O, n_slots, false);
+  e.p[KIND_GU] = plan_proj(h, KIND_GU, n_slots, true);
+  e.p[KIND_DN] = plan_proj(h, KIND_DN, n_slots, false);
+  if (h->step_plans.size() >= 16) h->step_plans.erase(h->step_plans.begin());
+  h->step_plans.push_back(e);
+  return h->step_plans.back();
+}
+
+template <int EPI>
+void launch_proj(tabed_handle* h, int kind, int layer, int n_slots, const ProjPlan& p, ProjArgs a) {
+  const tabed_handle::TcKind& t = h->tck[kind];
+  a.a_packed = h->tc_w + h->tc_off[kind] + (size_t)layer * h->tc_layer_stride;
+  a.k_chunks = t.k_chunks; a.ks = p.ks; a.cps = p.cps; a.n_stages = p.n_stages; a.recv_off = p.recv_off;
+  a.slots = h->slots; a.n_slots = n_slots; a.n_pad = p.n_pad; a.err = h->err;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(t.m_tiles * p.ks), (unsigned)p.n_tiles); cfg.blockDim = dim3(kTcThreads);
+  cfg.dynamicSmemBytes = p.smem; cfg.stream = h->stream;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)p.ks; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at; cfg.numAttrs = 2;
+  cudaLaunchKernelEx(&cfg, k_proj_tc<EPI>, a);
+  h->launches++;
+}
+
+template <int HD>
+void launch_prompt_attn(tabed_handle* h, int layer, int n, int act_npad, int act_chunks) {
+  PromptAttnArgs a{};
+  a.qkv = h->qkv; a.qkv_w = h->qkv_w; a.slots = h->slots; a.n = n;
+  a.kc = reinterpret_cast<const __nv_bfloat16*>(h->kc); a.vc = reinterpret_cast<const __nv_bfloat16*>(h->vc);
+  a.H = h->H; a.Hkv = h->Hkv; a.layer = layer; a.L = h->L; a.cap = h->cap; a.scale = 1.0f / sqrtf((float)h->hd);
+  a.act_out = h->tc_act; a.act_npad = act_npad; a.act_chunks = act_chunks;
+  TABED_LAUNCH_PDL(h, k_prompt_attn<HD>, dim3((n + kPaQ - 1) / kPaQ, h->H), kPaGroup * prompt_attn_groups(HD), prompt_attn_smem(HD), a);
+}
+
+// One shared-weight decoder step over `n_slots` slots with the projections on the tensor cores: 5 launches a layer.
+// logits_out null (prompts): only the caches are wanted, so the last layer ends with its appended K, V.
 void run_step_tc(tabed_handle* h, StepArgs sa, int n_slots, int max_pos, float* logits_out) {
   using bf = __nv_bfloat16;
-  sa.R = h->R; sa.m = h->m; sa.d = h->d; sa.G = h->G;
+  const int d = h->d, n_ss = proj_n_ss(h);
+  const bool prompt = sa.mode == STEP_PREFILL;
+  sa.R = h->R; sa.m = h->m; sa.d = d; sa.G = h->G;
   sa.kv_len = h->kv_len; sa.pending = h->pending;
   sa.slots = h->slots; sa.last_slot = h->last_slot; sa.x = h->x; sa.err = h->err; sa.kv_capacity = h->cap;
+  sa.ss = h->tc_ss_a; sa.n_ss = n_ss;
   TABED_LAUNCH_PDL(h, k_begin_step<bf>, n_slots, 128, 0, sa, reinterpret_cast<const bf*>(h->embed));
-  const size_t S2 = (size_t)h->slot_cap;
-  const int d = h->d, HD = h->H * h->hd, F = h->F;
-  struct Grp { int s0, n; };
-  std::vector<Grp> groups;                       // up to 256 slots share one pass over the weights
-  for (int g0 = 0; g0 < n_slots; g0 += kTcMaxN) groups.push_back({g0, std::min(kTcMaxN, n_slots - g0)});
-  auto prep_row = [&](const Grp& g, const float* partial, int ks, size_t slab, int write_back, const void* gain, const int* src, const SlotDesc* slots) {
+  const tabed_handle::StepPlan& plan = step_plan(h, n_slots);
+  const ProjPlan &pq = plan.p[KIND_QKV], &po = plan.p[KIND_O], &pg = plan.p[KIND_GU], &pd = plan.p[KIND_DN];
+  // act operand of a projection that starts with an RMSNorm of the residual: taken in its prologue, or packed first
+  auto normed = [&](ProjArgs& a, const ProjPlan& p, const float* ss, const void* gain) {
+    a.gain = reinterpret_cast<const bf*>(gain); a.eps = h->cfg.rms_eps; a.d = d; a.ss_in = ss; a.n_ss = n_ss;
+    if (p.norm) { a.x = h->x; return; }
     PrepRowArgs P{};
-    P.x = h->x; P.d = d; P.partial = partial; P.ks = partial ? ks : 0; P.slab = slab; P.src_slot = src; P.slots = slots;
-    P.gain = reinterpret_cast<const bf*>(gain); P.eps = h->cfg.rms_eps; P.slot0 = g.s0; P.n = g.n; P.n_pad = (g.n + 15) / 16 * 16;
-    P.write_back = write_back; P.dst = h->tc_act;
-    TABED_LAUNCH_PDL(h, k_prep_row, g.n, 256, 0, P);
+    P.x = h->x; P.d = d; P.ss = ss; P.n_ss = n_ss; P.slots = h->slots;
+    P.gain = a.gain; P.eps = a.eps; P.n_pad = p.n_pad; P.k_chunks = h->tck[KIND_QKV].k_chunks; P.dst = h->tc_act;
+    TABED_LAUNCH_PDL(h, k_prep_row, n_slots, 128, 0, P);
+    a.b_packed = h->tc_act;
   };
   for (int l = 0; l < h->L; ++l) {
     {
       ProfScope ps(h, TABED_PROF_QKV);
-      for (const Grp& g : groups) {
-        prep_row(g, l == 0 ? nullptr : h->tc_pd, h->tck[KIND_DN].ks, S2 * d, 1, h->norm1[l], nullptr, h->slots);
-        launch_gemm_tc(h, KIND_QKV, l, g.n, h->tc_pq + (size_t)g.s0 * h->qkv_w, S2 * h->qkv_w, h->slots + g.s0, h->qkv_w);
-      }
-      // the split-K slabs of the projection are summed by the kernel that rotates q, k and appends k, v
-      TABED_LAUNCH_PDL(h, k_rope_append<bf>, n_slots, 512, 0, h->qkv, h->slots, h->H, h->Hkv, h->hd, h->rope_cos, h->rope_sin,
-                   reinterpret_cast<bf*>(h->kc), reinterpret_cast<bf*>(h->vc), l, h->L, h->cap,
-                   (const float*)h->tc_pq, h->tck[KIND_QKV].ks, S2 * h->qkv_w);
+      ProjArgs a{};
+      normed(a, pq, h->tc_ss_a, h->norm1[l]);
+      a.rows = h->qkv_w; a.qkv = h->qkv; a.rope_cos = h->rope_cos; a.rope_sin = h->rope_sin;
+      a.kc = reinterpret_cast<bf*>(h->kc); a.vc = reinterpret_cast<bf*>(h->vc);
+      a.H = h->H; a.Hkv = h->Hkv; a.hd = h->hd; a.layer = l; a.L = h->L; a.cap = h->cap;
+      launch_proj<PROJ_QKV>(h, KIND_QKV, l, n_slots, pq, a);
     }
-    bool attn_wrote_act = false;
+    if (!logits_out && l == h->L - 1) break;
     {
       ProfScope ps(h, TABED_PROF_ATTENTION);       // the attention kernel(s) alone on this path
-      // one slot group: the attention kernel can leave its output as the O projection's operand blocks
-      const bool one = groups.size() == 1;
-      launch_attention_t<bf>(h, l, n_slots, max_pos, one ? h->tc_act : nullptr, one ? (groups[0].n + 15) / 16 * 16 : 0, &attn_wrote_act);
+      if (!prompt) launch_attention_t<bf>(h, l, n_slots, max_pos, h->tc_act, po.n_pad, h->tck[KIND_O].k_chunks);
+      else if (h->hd == 32) launch_prompt_attn<32>(h, l, n_slots, po.n_pad, h->tck[KIND_O].k_chunks);
+      else if (h->hd == 64) launch_prompt_attn<64>(h, l, n_slots, po.n_pad, h->tck[KIND_O].k_chunks);
+      else launch_prompt_attn<128>(h, l, n_slots, po.n_pad, h->tck[KIND_O].k_chunks);
     }
     {
       ProfScope ps(h, TABED_PROF_OPROJ);
-      for (const Grp& g : groups) {
-        const int n_pad = (g.n + 15) / 16 * 16;
-        if (!attn_wrote_act)
-          TABED_LAUNCH_PDL(h, k_prep_act, h->tck[KIND_O].k_chunks, 256, 0, h->attn_out + (size_t)g.s0 * HD, HD, g.n, n_pad, HD,
-                     (const float*)nullptr, (const bf*)nullptr, h->tc_act);
-        launch_gemm_tc(h, KIND_O, l, g.n, h->tc_po + (size_t)g.s0 * d, S2 * d, h->slots + g.s0, d);
-      }
+      ProjArgs a{};
+      a.b_packed = h->tc_act; a.rows = d; a.x_out = h->x; a.ss_out = h->tc_ss_m; a.n_ss = n_ss;
+      launch_proj<PROJ_RESID>(h, KIND_O, l, n_slots, po, a);
     }
     {
       ProfScope ps(h, TABED_PROF_GATEUP);
-      for (const Grp& g : groups) {
-        prep_row(g, h->tc_po, h->tck[KIND_O].ks, S2 * d, 1, h->norm2[l], nullptr, h->slots);
-        launch_gemm_tc(h, KIND_GU, l, g.n, h->tc_pgu + (size_t)g.s0 * 2 * F, S2 * 2 * F, h->slots + g.s0, 2 * F);
-      }
+      ProjArgs a{};
+      normed(a, pg, h->tc_ss_m, h->norm2[l]);
+      a.act_out = h->tc_mid; a.act_npad = pd.n_pad; a.act_chunks = h->tck[KIND_DN].k_chunks;
+      launch_proj<PROJ_SWIGLU>(h, KIND_GU, l, n_slots, pg, a);
     }
     {
       ProfScope ps(h, TABED_PROF_DOWN);
-      for (const Grp& g : groups) {
-        const int n_pad = (g.n + 15) / 16 * 16;
-        TABED_LAUNCH_PDL(h, k_swiglu_prep, dim3(h->tck[KIND_DN].k_chunks, g.n), kTcKC / 8, 0, h->tc_pgu, h->tck[KIND_GU].ks, S2 * 2 * F, F,
-                     h->slots, g.s0, n_pad, h->tc_act);
-        launch_gemm_tc(h, KIND_DN, l, g.n, h->tc_pd + (size_t)g.s0 * d, S2 * d, h->slots + g.s0, d);
-      }
+      ProjArgs a{};
+      a.b_packed = h->tc_mid; a.rows = d; a.x_out = h->x; a.ss_out = h->tc_ss_a; a.n_ss = n_ss;
+      launch_proj<PROJ_RESID>(h, KIND_DN, l, n_slots, pd, a);
     }
   }
   if (logits_out) {
     ProfScope ps(h, TABED_PROF_LM_HEAD);
-    for (int r0 = 0; r0 < h->R; r0 += kTcMaxN) {
-      const Grp g{r0, std::min(kTcMaxN, h->R - r0)};
-      prep_row(g, h->tc_pd, h->tck[KIND_DN].ks, S2 * d, 0, h->final_norm, h->last_slot, nullptr);
-      launch_gemm_tc(h, KIND_LM, 0, g.n, logits_out + (size_t)r0 * h->V, 0, nullptr, h->V);
-    }
+    PrepRowArgs P{};
+    const int n_pad = tc_n_pad(h->R);
+    P.x = h->x; P.d = d; P.ss = h->tc_ss_a; P.n_ss = n_ss; P.src_slot = h->last_slot;
+    P.gain = reinterpret_cast<const bf*>(h->final_norm); P.eps = h->cfg.rms_eps; P.n_pad = n_pad; P.k_chunks = h->tck[KIND_LM].k_chunks;
+    P.dst = h->tc_act;
+    TABED_LAUNCH_PDL(h, k_prep_row, h->R, 128, 0, P);
+    for (int r0 = 0, t = 0; r0 < h->R; r0 += n_pad, ++t)
+      launch_lm_head_tc(h, h->tc_act + (size_t)t * P.k_chunks * tc_block_bytes(n_pad), std::min(n_pad, h->R - r0), n_pad, logits_out + (size_t)r0 * h->V);
   }
 }
 
@@ -913,10 +1029,10 @@ int tabed_init(const tabed_config* cfg, const tabed_weights* wts, tabed_handle**
     const size_t SC = (c.dtype == TABED_DTYPE_BF16) ? std::max<size_t>(2 * R, kPrefillChunk) : 2 * R;
     h->slot_cap = (int)SC;
     A(&h->kv_len, R); A(&h->slots, SC); A(&h->last_slot, R);
-    A(&h->x, SC * h->d); A(&h->qkv, SC * h->qkv_w); A(&h->attn_out, SC * h->H * h->hd); A(&h->mid, SC * h->F);
-    A(&h->part_o, SC * h->H * (size_t)h->max_splits * h->hd); A(&h->part_ml, SC * h->H * (size_t)h->max_splits * 2);
+    A(&h->x, SC * h->d); A(&h->qkv, SC * h->qkv_w); A(&h->attn_out, 2 * R * h->H * h->hd); A(&h->mid, 2 * R * h->F);
+    A(&h->part_o, 2 * R * h->H * (size_t)h->max_splits * h->hd); A(&h->part_ml, 2 * R * h->H * (size_t)h->max_splits * 2);
     A(&h->logits_own, G * R * V);
-    A(&h->attn_tickets, SC * h->Hkv);
+    A(&h->attn_tickets, 2 * R * h->Hkv);
     if (c.dtype == TABED_DTYPE_BF16 && h->hd == kAtcHd && h->H / h->Hkv <= kMaxGroup && rc == TABED_OK) {
       // TMA descriptors of the caches seen as [all rows of all (row, layer, head)][64] bf16, tiles of 128 rows, 128-byte swizzle
       typedef CUresult (*EncodeFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
@@ -926,7 +1042,7 @@ int tabed_init(const tabed_config* cfg, const tabed_weights* wts, tabed_handle**
       cudaDriverEntryPointQueryResult qres;
       const unsigned long long n_rows = (unsigned long long)R * h->L * h->Hkv * (unsigned long long)h->cap;
       if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &qres) == cudaSuccess && fn &&
-          qres == cudaDriverEntryPointSuccess && n_rows < (1ull << 31)) {
+          qres == cudaDriverEntryPointSuccess && n_rows < (1ull << 31) && h->cap <= kAtcMaxCap) {
         const cuuint64_t dims[2] = {(cuuint64_t)kAtcHd, (cuuint64_t)n_rows};
         const cuuint64_t strides[1] = {(cuuint64_t)kAtcHd * 2};
         const cuuint32_t box[2] = {(cuuint32_t)kAtcHd, (cuuint32_t)kAtcSplit};
@@ -1548,7 +1664,7 @@ int tabed_debug_gemm_tc(const void* w, const float* act, int32_t rows, int32_t K
     rc = TABED_ERR_CUDA;
   if (rc == TABED_OK) {
     k_pack_tc<<<dim3(k_chunks, m_tiles), 256, 0, st>>>(reinterpret_cast<const __nv_bfloat16*>(w), rows, nullptr, 0, nullptr, 0, K, k_chunks, a_p);
-    k_prep_act<<<k_chunks, 256, 0, st>>>(act, K, n, n_pad, K, nullptr, nullptr, b_p);
+    k_prep_act<<<k_chunks, 256, 0, st>>>(act, K, n, n_pad, K, b_p);
     TcGemmArgs G{};
     G.a_packed = a_p; G.b_packed = b_p; G.partial = part; G.slab = (size_t)n * rows; G.rows_total = rows; G.rows_valid = rows; G.n_pad = n_pad; G.n_slots = n;
     G.k_chunks = k_chunks; G.ks = ks; G.cps = cps; G.err = err;

@@ -1,0 +1,65 @@
+"""The fused layer projections and the prompt attention at the sizes where their tiles end: a prompt fed in chunks through
+the tensor-core kernels, and a decoder step of many rows, against the same work one kernel per operation (each of the two is
+within the checker's bound, so they differ by at most twice that bound)."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2601_20357_b200 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+if torch.cuda.is_available():
+    import gpu_harness as H
+    from paper_2601_20357_b200 import binding as TB
+
+
+def _workload(B, m, heads, kv_heads, hd, ffn, cap):
+    cfg = W.DrafterCfg(2, heads * hd, heads, kv_heads, ffn, 1003, "bf16")
+    return W.Workload(name=f"proj{heads}x{hd}", config_id=91, drafter=cfg, n_inputs=m, n_requests=B, gamma=2, window_h=4, rounds=1,
+                      policy=W.POLICY_STATIC, prefixes=((("tokens", 1),),) * m, kv_capacity=cap, alpha=(1.0 / m,) * m)
+
+
+def _handle(wl, weights):
+    return TB.Tabed(n_inputs=wl.n_inputs, n_requests=wl.n_requests, gamma=wl.gamma, window_h=wl.window_h, policy=wl.policy,
+                    vocab=wl.drafter.vocab, drafter=wl.drafter, weights=weights, kv_capacity=wl.kv_capacity)
+
+
+def _logits_after(wl, weights, path, lengths, seed):
+    """Logits of one decoder step after every row's prompt (token part, then embedding part) has been fed on `path`."""
+    g = _handle(wl, weights)
+    gen = torch.Generator(device="cuda").manual_seed(seed)
+    g.select_path(path)
+    for row, (n_tok, n_emb) in enumerate(lengths):
+        if n_tok:
+            g.prefill_tokens(row, torch.randint(0, wl.drafter.vocab, (n_tok,), generator=gen, device="cuda", dtype=torch.int32))
+        if n_emb:
+            g.prefill_embeds(row, torch.randn((n_emb, wl.drafter.d_model), generator=gen, device="cuda"))
+    tok = torch.randint(0, wl.drafter.vocab, (wl.n_requests,), generator=gen, device="cuda", dtype=torch.int32)
+    out = torch.empty((wl.n_rows, wl.drafter.vocab), device="cuda")
+    g.decode_step(tok, out)
+    torch.cuda.synchronize()
+    assert g.last_device_error() == 0
+    g.destroy()
+    return out.cpu().numpy()
+
+
+@pytest.mark.parametrize("heads,kv_heads,hd,ffn", [(4, 4, 64, 640), (7, 1, 64, 520), (11, 11, 32, 704), (3, 3, 128, 776)])
+@pytest.mark.parametrize("lengths", [((1, 0), (63, 1), (64, 65)), ((0, 129), (255, 2), (1030, 0))])
+def test_prompt_chunks_agree_with_one_position_at_a_time(heads, kv_heads, hd, ffn, lengths):
+    wl = _workload(1, 3, heads, kv_heads, hd, ffn, 1040)
+    weights = TB.weights_to_device(wl.drafter, W.make_weights(wl), torch.device("cuda", 0))
+    a = _logits_after(wl, weights, TB.PATH_TENSOR_CORE, lengths, 5)
+    b = _logits_after(wl, weights, TB.PATH_PER_OP, lengths, 5)
+    assert np.max(np.abs(a - b)) <= 2 * H.logit_tols(wl)[0]
+
+
+@pytest.mark.parametrize("B,m", [(1, 1), (5, 3), (11, 3), (43, 3), (129, 2)])
+def test_rows_at_tile_edges_agree_with_per_operation_step(B, m):
+    """1, 15, 33, 129 and 258 rows: one tile and several, whole and ragged (the plan of a projection depends on the count)."""
+    wl = _workload(B, m, 6, 2, 64, 520, 40)
+    weights = TB.weights_to_device(wl.drafter, W.make_weights(wl), torch.device("cuda", 0))
+    lengths = [(1 + r % 7, 0) for r in range(wl.n_rows)]
+    a = _logits_after(wl, weights, TB.PATH_TENSOR_CORE, lengths, 6)
+    b = _logits_after(wl, weights, TB.PATH_PER_OP, lengths, 6)
+    assert np.max(np.abs(a - b)) <= 2 * H.logit_tols(wl)[0]
