@@ -318,6 +318,9 @@ __device__ __forceinline__ int req_best_of(const ReqCtx& c, const ReqShared& S, 
 // ------------------------------------------------------------------------------------------------
 struct EnsembleArgs {
   int V, m, greedy, slice;
+  int steps;                                    // cluster (b, i) takes step i of request b (the caller's own logits: all steps of a round
+                                                // are known at once; else 1)
+  long long logits_step;                        // ... whose operands are this / m V / V / D elements further on
   int D;                                        // candidates per step (1: a plain chain); candidate c uses u[.. + c]
   int* cand; int cand_stride;                   // optional: all candidates, cand[b * cand_stride + c] (-1: none left)
   const float* logits;
@@ -338,12 +341,12 @@ __global__ void __launch_bounds__(kReqThreads, 2) k_ensemble_req(const EnsembleA
   cg::cluster_group cluster = cg::this_cluster();
   __shared__ ReqShared S;
   const ReqCtx c = req_ctx(cluster, A.V, A.slice);
-  const int b = blockIdx.x / c.CS, m = A.m, V = A.V;
+  const int unit = blockIdx.x / c.CS, b = unit / A.steps, step = unit - b * A.steps, m = A.m, V = A.V;
   float* ebuf = A.ebuf_pitch > 0 ? reinterpret_cast<float*>(req_dyn_smem) : nullptr;
   const int epitch = A.ebuf_pitch;
   pdl_wait();
-  const float* lg = A.logits + (long long)b * m * V;
-  const bool vec = req_vec_ok(A.logits, V);
+  const float* lg = A.logits + step * A.logits_step + (long long)b * m * V;
+  const bool vec = req_vec_ok(A.logits, V) && (A.logits_step & 3) == 0;
   req_row_maxima(cluster, c, S, lg, V, m, vec, ebuf, epitch);
   req_row_sums(cluster, c, S, lg, V, m, vec, ebuf, epitch);
   // (the loop over the inputs below is a real loop - the kernel's code runs once per CTA, so its size is what
@@ -354,8 +357,8 @@ __global__ void __launch_bounds__(kReqThreads, 2) k_ensemble_req(const EnsembleA
     S.par[2][c.tid] = A.w[b * m + c.tid];
   }
   __syncthreads();
-  float* q_row = A.q_out + (long long)b * A.q_req_stride;
-  float* qk_b = A.qk_out ? A.qk_out + (long long)b * A.qk_req_stride : nullptr;
+  float* q_row = A.q_out + (long long)b * A.q_req_stride + (long long)step * V;
+  float* qk_b = A.qk_out ? A.qk_out + (long long)b * A.qk_req_stride + (long long)step * m * V : nullptr;
   const bool vec_q = req_vec_ok(A.q_out, A.q_req_stride) && (V & 3) == 0;
   const bool vec_qk = A.qk_out && req_vec_ok(A.qk_out, A.qk_req_stride) && (V & 3) == 0;
   unsigned long long mass = 0;
@@ -395,9 +398,9 @@ __global__ void __launch_bounds__(kReqThreads, 2) k_ensemble_req(const EnsembleA
   const int D = A.D;
   int chosen[kReqMaxWidth] = {-1, -1, -1, -1};
   auto emit = [&](int cnd, int y) {
-    if (cnd == 0) A.out0[b * A.out0_stride] = y;
-    if (A.out1) A.out1[b * A.out1_stride + cnd] = y;
-    if (A.cand) A.cand[b * A.cand_stride + cnd] = y;
+    if (cnd == 0) A.out0[b * A.out0_stride + step] = y;
+    if (A.out1) A.out1[b * A.out1_stride + step * D + cnd] = y;
+    if (A.cand) A.cand[b * A.cand_stride + step * D + cnd] = y;
   };
   if (A.greedy) {
 #pragma unroll 1
@@ -458,7 +461,7 @@ __global__ void __launch_bounds__(kReqThreads, 2) k_ensemble_req(const EnsembleA
 #pragma unroll 1
   for (int cnd = 0; cnd < D; ++cnd) {
     int y = 0, status = 0;
-    const bool mine = req_draw(c, S, 0, A.u[b * A.u_stride + cnd], mass, t_lo, t_hi, mass_left, &y, &status);
+    const bool mine = req_draw(c, S, 0, A.u[b * A.u_stride + step * D + cnd], mass, t_lo, t_hi, mass_left, &y, &status);
     if (status == 1) {
       // nothing (left) to draw from: an error for the chain's own token, "no candidate" for a sibling
       if (c.rank == 0 && c.tid == 0) {
