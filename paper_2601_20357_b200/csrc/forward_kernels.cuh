@@ -177,6 +177,8 @@ __global__ void __launch_bounds__(kGemvThreads) k_gemv(GemvArgs A) {
   extern __shared__ __align__(16) float xs[];          // [NS][K]
   __shared__ float red[kGemvWarps];
   constexpr int EL = Elem<T>::kPerVec;
+  pdl_trigger();
+  pdl_wait();
   const int K = A.K;
   const int slot_base = blockIdx.y * NS;
   const int ns = min(NS, A.n_slots - slot_base);
@@ -315,6 +317,8 @@ template <typename T>
 __global__ void k_rope_append(float* __restrict__ qkv, const SlotDesc* __restrict__ slots, int H, int Hkv, int hd,
                               const float* __restrict__ rope_cos, const float* __restrict__ rope_sin,
                               T* __restrict__ kc, T* __restrict__ vc, int layer, int L, int cap) {
+  pdl_trigger();
+  pdl_wait();
   const int s = blockIdx.x;
   const SlotDesc sd = slots[s];
   if (!sd.active) return;
@@ -366,6 +370,8 @@ k_attn_partial(const float* __restrict__ qkv, const SlotDesc* __restrict__ slots
   constexpr int LPR = HD / EL;                 // lanes per cache row
   constexpr int PPW = 32 / LPR;                // positions per warp pass
   constexpr int NW = kAttnThreads / 32;
+  pdl_trigger();
+  pdl_wait();
   const int s = blockIdx.z, g = blockIdx.y, split = blockIdx.x;
   const SlotDesc sd = slots[s];
   if (!sd.active) return;
