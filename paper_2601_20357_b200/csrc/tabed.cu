@@ -109,8 +109,7 @@ struct tabed_handle {
   unsigned char* packed = nullptr;
   unsigned long long* trace = nullptr; int trace_stride = 0; bool trace_on = false; int trace_cta = 0;
   // tensor-core projections for many rows (bf16 drafter, more than 8 slots per step)
-  bool tc_ok = false;                        // tcgen05 projections are set up (prefill in chunks; drafting when tc_auto)
-  bool tc_auto = false;                      // ... and are the automatic choice for drafting (no persistent kernel)
+  bool tc_ok = false;                        // tcgen05 projections are set up: prompts, single steps, and rounds without the persistent kernel
   int slot_cap = 0;                          // slots the step buffers hold: 2R, or a prefill chunk if that is more
   struct TcKind { int rows, K, m_tiles, k_chunks; size_t bytes; };
   TcKind tck[5]{};                  // KIND_QKV, KIND_O, KIND_GU (tiles of 64 gate + 64 up rows), KIND_DN, KIND_LM
@@ -663,7 +662,6 @@ int setup_tc(tabed_handle* h) {
   }
   if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(h->stream) != cudaSuccess) return TABED_ERR_CUDA;
   h->tc_ok = true;
-  h->tc_auto = !h->persist_ok;            // measured faster than one kernel per operation from 6 rows on (1.46 vs 2.20 ms)
   return TABED_OK;
 }
 
@@ -870,9 +868,11 @@ int read_clear_device_error(int* err_dev, cudaStream_t st, int* bits_out) {
   return TABED_OK;
 }
 
-// drafting steps outside the persistent kernel: tensor-core projections when chosen (or automatic with many rows)
+// Decoder steps outside the persistent kernel: tensor-core projections when chosen or automatic.  With five launches a layer
+// they are the faster way for any number of rows (prompt and one step of 3 rows of the 4-layer drafter 1148 -> 1048 us, of 4
+// rows of the 12-layer one 7644 -> 7073, against one kernel per operation for the step).
 bool use_tc(const tabed_handle* h) {
-  return h->tc_ok && (h->path_sel == TABED_PATH_TENSOR_CORE || (h->path_sel == TABED_PATH_AUTO && h->tc_auto));
+  return h->tc_ok && (h->path_sel == TABED_PATH_TENSOR_CORE || h->path_sel == TABED_PATH_AUTO);
 }
 
 int max_len_ub(const tabed_handle* h) {
@@ -1504,7 +1504,7 @@ int tabed_current_path(const tabed_handle* h) {
   if (h->path_sel == TABED_PATH_PER_OP) return TABED_PATH_PER_OP;
   if (h->path_sel == TABED_PATH_TENSOR_CORE) return TABED_PATH_TENSOR_CORE;
   if (h->path_sel == TABED_PATH_PERSISTENT) return TABED_PATH_PERSISTENT;
-  return h->persist_ok ? TABED_PATH_PERSISTENT : (h->tc_auto ? TABED_PATH_TENSOR_CORE : TABED_PATH_PER_OP);
+  return h->persist_ok ? TABED_PATH_PERSISTENT : (h->tc_ok ? TABED_PATH_TENSOR_CORE : TABED_PATH_PER_OP);
 }
 
 int tabed_debug_trace(tabed_handle* h, int32_t on) {
