@@ -1,15 +1,17 @@
 // Causal attention of a prompt's positions (all of one cache row) over that row's bf16 cache, K and V of the positions
 // themselves already appended: the chunk of positions that one pass of the tensor-core projections feeds.
 //
-// A CTA takes 64 positions of one query head and walks the cache in tiles of 64 positions (cp.async, two buffers, 16-byte
-// pieces XOR-swizzled so that every ldmatrix is conflict-free); a warp owns 16 positions.  The tiles are dealt to two or four
-// groups of four warps (a tile's chain of products and softmax is 1.8 us for a lone group, and a short prompt fills a
-// fraction of the SMs); their states meet in shared memory at the end.  scores = Q K^T and out += P V on
-// mma.sync m16n8k16 (bf16 x bf16 -> fp32): q is a bf16 value already, the softmax weights are split into a bf16 head and a
-// bf16 remainder (two products), so products are exact to ~2^-17 and sums are fp32, as in the decode kernels.  A prompt of
-// 576 positions and 12 heads is 2 GFLOP against 0.9 MB of cache per head: neither roofline is near, what counts is that the
-// K, V tiles are shared by 64 positions (the decode kernel reads the cache once per position: 66 us for 256 positions of a
-// 768-wide layer, this one 14 for 576).  The longest CTAs (last positions) start first.
+// A CTA takes 16 QW positions of one query head and walks the cache in tiles of T positions (cp.async, two buffers, 16-byte
+// pieces XOR-swizzled so that every ldmatrix is conflict-free); a warp owns 16 positions.  The tiles are dealt to NG groups of
+// QW warps (a tile's chain of products and softmax is 1.8 us for a lone group); their states meet in shared memory at the
+// end.  scores = Q K^T and out += P V on mma.sync m16n8k16 (bf16 x bf16 -> fp32): q is a bf16 value already, the softmax
+// weights are split into a bf16 head and a bf16 remainder (two products), so products are exact to ~2^-17 and sums are fp32,
+// as in the decode kernels.  A prompt of 576 positions and 12 heads is 2 GFLOP against 0.9 MB of cache per head: neither
+// roofline is near, what counts is that the K, V tiles are shared by the CTA's positions (the decode kernel reads the cache
+// once per position: 66 us for 256 positions of a 768-wide layer, this one 14 for 576).  The longest CTAs (last positions)
+// start first.  Short prompts would leave most SMs idle with 64 positions a CTA (128 positions x 12 heads: 24 CTAs, whose
+// products then wait for one another on the tensor pipe): where these CTAs fill at most half of the SMs, 32 positions and
+// tiles of 32 in eight groups are taken.
 #pragma once
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -19,11 +21,10 @@
 
 namespace tabed {
 
-constexpr int kPaQ = 64;              // positions per CTA (16 per warp)
-constexpr int kPaT = 64;              // cache positions per tile
-constexpr int kPaGroup = kPaQ / 16 * 32;      // threads of a group
-__host__ __device__ constexpr int prompt_attn_groups(int hd) { return hd <= 64 ? 4 : 2; }
-__host__ __device__ constexpr size_t prompt_attn_smem(int hd) { return (size_t)prompt_attn_groups(hd) * 4 * kPaT * hd * 2; }      // two buffers of K and V each
+// groups of a CTA: 16 warps in all, 8 for 128-wide heads
+template <int HD, int QW> __host__ __device__ constexpr int prompt_attn_groups() { return (HD <= 64 ? 16 : 8) / QW; }
+// two buffers of K and V per group
+template <int HD, int QW, int T> __host__ __device__ constexpr size_t prompt_attn_smem() { return (size_t)prompt_attn_groups<HD, QW>() * 4 * T * HD * 2; }
 
 struct PromptAttnArgs {
   const float* qkv; int qkv_w;                 // [n][qkv_w] rotated q
@@ -38,12 +39,12 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
 }
 
-// grid (tiles of kPaQ positions, H)
-template <int HD>
-__global__ void __launch_bounds__(kPaGroup * prompt_attn_groups(HD), 1) k_prompt_attn(const PromptAttnArgs A) {
+// grid (tiles of 16 QW positions, H)
+template <int HD, int QW, int T>
+__global__ void __launch_bounds__(QW * 32 * prompt_attn_groups<HD, QW>(), 1) k_prompt_attn(const PromptAttnArgs A) {
   extern __shared__ __align__(128) unsigned char pa_smem[];
-  constexpr int NG = prompt_attn_groups(HD);
-  __shared__ float s_ml[NG][4][2][16];         // (max, sum) of every position by group
+  constexpr int NG = prompt_attn_groups<HD, QW>(), kPaQ = 16 * QW, kPaT = T, kPaGroup = 32 * QW;
+  __shared__ float s_ml[NG][QW][2][16];         // (max, sum) of every position by group
   constexpr int PIECES = HD / 8;               // 16-byte pieces of a cache row
   constexpr int KK = HD / 16, NT = HD / 8;
   constexpr unsigned FULL = 0xffffffffu;
@@ -172,7 +173,7 @@ __global__ void __launch_bounds__(kPaGroup * prompt_attn_groups(HD), 1) k_prompt
   __syncthreads();
   float4* st = reinterpret_cast<float4*>(pa_smem);
 #pragma unroll
-  for (int j = 0; j < NT; ++j) st[((grp * 4 + warp) * NT + j) * 32 + lane] = make_float4(o[j][0], o[j][1], o[j][2], o[j][3]);
+  for (int j = 0; j < NT; ++j) st[((grp * QW + warp) * NT + j) * 32 + lane] = make_float4(o[j][0], o[j][1], o[j][2], o[j][3]);
   if (t4 == 0) {
     s_ml[grp][warp][0][g] = m_run[0]; s_ml[grp][warp][0][g + 8] = m_run[1];
     s_ml[grp][warp][1][g] = l_run[0]; s_ml[grp][warp][1][g + 8] = l_run[1];
@@ -191,12 +192,11 @@ __global__ void __launch_bounds__(kPaGroup * prompt_attn_groups(HD), 1) k_prompt
   }
   const int r0 = q0 + warp * 16 + g, r1 = r0 + 8;
 #pragma unroll
-  for (int jj = 0; jj < NT / NG; ++jj) {
-    const int j = grp * (NT / NG) + jj;
+  for (int j = grp; j < NT; j += NG) {
     float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
 #pragma unroll
     for (int i = 0; i < NG; ++i) {
-      const float4 x = st[((i * 4 + warp) * NT + j) * 32 + lane];
+      const float4 x = st[((i * QW + warp) * NT + j) * 32 + lane];
       v.x = fmaf(f[0][i], x.x, v.x); v.y = fmaf(f[0][i], x.y, v.y); v.z = fmaf(f[1][i], x.z, v.z); v.w = fmaf(f[1][i], x.w, v.w);
     }
     const int k = head * HD + j * 8 + 2 * t4;

@@ -622,8 +622,10 @@ int setup_tc(tabed_handle* h) {
   if (std::max(h->tc_smem, kProjMaxSmem) > (size_t)prop.sharedMemPerBlockOptin) return TABED_OK;
   auto smem_attr = [](auto kern, size_t bytes) { return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess; };
   if (!smem_attr(k_gemm_tc, h->tc_smem) || !smem_attr(k_proj_tc<PROJ_QKV>, kProjMaxSmem) || !smem_attr(k_proj_tc<PROJ_RESID>, kProjMaxSmem) ||
-      !smem_attr(k_proj_tc<PROJ_SWIGLU>, kProjMaxSmem) || !smem_attr(k_prompt_attn<32>, prompt_attn_smem(32)) ||
-      !smem_attr(k_prompt_attn<64>, prompt_attn_smem(64)) || !smem_attr(k_prompt_attn<128>, prompt_attn_smem(128)))
+      !smem_attr(k_proj_tc<PROJ_SWIGLU>, kProjMaxSmem) || !smem_attr(k_prompt_attn<32, 4, 64>, prompt_attn_smem<32, 4, 64>()) ||
+      !smem_attr(k_prompt_attn<64, 4, 64>, prompt_attn_smem<64, 4, 64>()) || !smem_attr(k_prompt_attn<128, 4, 64>, prompt_attn_smem<128, 4, 64>()) ||
+      !smem_attr(k_prompt_attn<32, 2, 32>, prompt_attn_smem<32, 2, 32>()) || !smem_attr(k_prompt_attn<64, 2, 32>, prompt_attn_smem<64, 2, 32>()) ||
+      !smem_attr(k_prompt_attn<128, 2, 32>, prompt_attn_smem<128, 2, 32>()))
     return TABED_ERR_CUDA;
   // Clusters of a projection that the device keeps resident at once (an SM group does not divide evenly into every size: 148
   // SMs hold 74 pairs but 45 threes).  The occupancy calculator gives every kernel with tensor memory the SM to itself; with
@@ -768,7 +770,9 @@ void launch_prompt_attn(tabed_handle* h, int layer, int n, int act_npad, int act
   a.kc = reinterpret_cast<const __nv_bfloat16*>(h->kc); a.vc = reinterpret_cast<const __nv_bfloat16*>(h->vc);
   a.H = h->H; a.Hkv = h->Hkv; a.layer = layer; a.L = h->L; a.cap = h->cap; a.scale = 1.0f / sqrtf((float)h->hd);
   a.act_out = h->tc_act; a.act_npad = act_npad; a.act_chunks = act_chunks;
-  TABED_LAUNCH_PDL(h, k_prompt_attn<HD>, dim3((n + kPaQ - 1) / kPaQ, h->H), kPaGroup * prompt_attn_groups(HD), prompt_attn_smem(HD), a);
+  auto go = [&](auto kern, int rows, int threads, size_t smem) { TABED_LAUNCH_PDL(h, kern, dim3((n + rows - 1) / rows, h->H), threads, smem, a); };
+  if (2 * ((n + 63) / 64) * h->H > h->n_sm) go(k_prompt_attn<HD, 4, 64>, 64, 128 * prompt_attn_groups<HD, 4>(), prompt_attn_smem<HD, 4, 64>());
+  else go(k_prompt_attn<HD, 2, 32>, 32, 64 * prompt_attn_groups<HD, 2>(), prompt_attn_smem<HD, 2, 32>());
 }
 
 // One shared-weight decoder step over `n_slots` slots with the projections on the tensor cores: 5 launches a layer.
