@@ -266,12 +266,19 @@ __device__ __forceinline__ bool req_draw(const ReqCtx& c, ReqShared& S, int whic
 #pragma unroll
   for (int i = 0; i < kReqWarps; ++i) if (i < c.warp) run += S.scan[i];
   if (run <= thr && thr < run + tmass) {
+    int y = 0x7fffffff;
 #pragma unroll 1
-    for (int v = t_lo; v < t_hi; ++v) {
-      const unsigned long long mv = mass_at(v);
-      run += mv;
-      if (run > thr && mv != 0ull) { S.result = v; break; }
+    for (int v = t_lo; v < t_hi && y == 0x7fffffff; v += 4) {      // four masses in flight (one trip to L2, not four)
+      unsigned long long mv[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) mv[j] = v + j < t_hi ? mass_at(v + j) : 0ull;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        run += mv[j];
+        if (run > thr && mv[j] != 0ull && y == 0x7fffffff) y = v + j;
+      }
     }
+    if (y != 0x7fffffff) S.result = y;
   }
   __syncthreads();
   const int y = S.result;
@@ -551,6 +558,14 @@ __global__ void __launch_bounds__(kReqThreads, 2) k_verify_req(const VerifyArgs 
   const float* q_b = A.q + (long long)b * A.q_req_stride;
   const bool vec = req_vec_ok(A.logits, V), vec_p = (V & 3) == 0;
   float* ebuf = A.ebuf_pitch > 0 ? reinterpret_cast<float*>(req_dyn_smem) : nullptr;
+  // the accept test's operands (they hang on the token) are requested beside the row
+  float ly = 0.0f, qy = 0.0f, uy = 0.0f;
+  if (c.rank == 0 && c.tid == 0 && i < G && !A.greedy) {
+    const int y = A.tokens[b * G + i];
+    ly = __ldg(lg + y);
+    qy = __ldg(q_b + (long long)i * V + y);
+    uy = A.u_accept[(b * G + i) * D];
+  }
   req_row_maxima(cluster, c, S, lg, V, 1, vec, ebuf, A.ebuf_pitch);
   req_row_sums(cluster, c, S, lg, V, 1, vec, ebuf, A.ebuf_pitch);
   const float mx = req_max_of(c, S, 0), sn = req_norm_of(c, S, 0);
@@ -582,10 +597,8 @@ __global__ void __launch_bounds__(kReqThreads, 2) k_verify_req(const VerifyArgs 
     int flag;
     if (A.greedy) flag = req_best_of(c, S, 0);
     else if (i < G) {
-      const int y = A.tokens[b * G + i];
-      const float py = __fdiv_rn(xexp(__fsub_rn(__ldg(lg + y), mx)), sn);          // the value stored in p_i[y]
-      const float qy = __ldg(q_b + (long long)i * V + y);
-      flag = (py >= qy) || (__fmul_rn(A.u_accept[(b * G + i) * D], qy) < py);
+      const float py = __fdiv_rn(xexp(__fsub_rn(ly, mx)), sn);                     // the value stored in p_i[y]
+      flag = (py >= qy) || (__fmul_rn(uy, qy) < py);
     } else flag = 1;
     A.row_flag[b * rows + i] = flag;
   }
@@ -610,12 +623,11 @@ __device__ __forceinline__ void verify_tail(cg::cluster_group& cluster, const Re
   float* p_b = A.p + (long long)b * Rt * V;
   const float* q_b = A.q + (long long)b * A.q_req_stride;
   const bool vec = req_vec_ok(A.logits, V), vec_p = (V & 3) == 0;
-  int a = 0;
-  for (; a < G; ++a) {
-    const int f = __ldcg(A.row_flag + b * rows + a);
-    if (A.greedy ? (f != A.tokens[b * G + a]) : (f == 0)) break;
-  }
+  // accepted prefix: lane = position, every flag in one trip to L2 (G <= 16)
+  const int my_flag = c.lane < rows ? __ldcg(A.row_flag + b * rows + c.lane) : 0;
   const float u = A.u_resid[b];
+  const bool stop = c.lane < G ? (A.greedy ? my_flag != A.tokens[b * G + c.lane] : my_flag == 0) : true;
+  const int a = min(G, __ffs(__ballot_sync(0xffffffffu, stop)) - 1);
   int t_lo, t_hi;
   req_thread_range(c, A.slice, &t_lo, &t_hi);
   int n_acc = a, sib = -1, z = 0, status = 0;
@@ -654,11 +666,11 @@ __device__ __forceinline__ void verify_tail(cg::cluster_group& cluster, const Re
   };
   if (A.greedy) {
     if (a < G) {
-      const int t = __ldcg(A.row_flag + b * rows + a);            // the target's token at the first depth that differs
+      const int t = __shfl_sync(0xffffffffu, my_flag, a);         // the target's token at the first depth that differs
       for (int cnd = 1; cnd < D; ++cnd) if (sib < 0 && A.cand[(b * G + a) * D + cnd] == t) sib = cnd;
       if (sib < 0) { z = t; mine = c.rank == 0; have_z = true; }
     } else {
-      z = __ldcg(A.row_flag + b * rows + G); mine = c.rank == 0; have_z = true;
+      z = __shfl_sync(0xffffffffu, my_flag, G); mine = c.rank == 0; have_z = true;
     }
   } else if (a < G) {
     // Recursive rejection over the depth's candidates.  Level l distributions are functions of (p_a, q_a) and of the
@@ -685,18 +697,19 @@ __device__ __forceinline__ void verify_tail(cg::cluster_group& cluster, const Re
       // this level's residual masses (per thread range) and the mass of q_level
       unsigned long long mr = 0, mq = 0;
 #pragma unroll 1
-      for (int v = t_lo; v < t_hi; ++v) {
-        float pl, ql;
-        elem(v, level, pl, ql);
-        mr += mass_of(resid_val(pl, ql));
-        mq += mass_of(ql);
+      for (int v = t_lo; v < t_hi; v += 4) {
+        float pl[4], ql[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) { pl[j] = ql[j] = 0.0f; if (v + j < t_hi) elem(v + j, level, pl[j], ql[j]); }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) { mr += mass_of(resid_val(pl[j], ql[j])); mq += mass_of(ql[j]); }      // (0 beyond the range)
       }
       const int buf = 2 * (level & 1);
       req_gather_mass2(cluster, c, S, mr, mq, buf);
       unsigned long long MR = 0, MQ = 0;
       for (unsigned r = 0; r < c.CS; ++r) { MR += S.all_mass[buf][r]; MQ += S.all_mass[buf + 1][r]; }
-      float px, qx;
-      elem(xs[level], level, px, qx);
+      float px = 0.0f, qx = 0.0f;
+      if (level + 1 < D) elem(xs[level], level, px, qx);           // (only asked for when a sibling may follow)
       const unsigned long long MQrest = MQ - mass_of(qx);
       const bool more = level + 1 < D && xs[level + 1] >= 0 && MR != 0ull && MQrest != 0ull;
       if (!more) {
@@ -925,38 +938,56 @@ __global__ void __launch_bounds__(kReqThreads, 2) k_update_req(const UpdateArgs 
 // One warp per request: lane kd carries deviation index kd through the window (its running sum stays in a
 // register), then lane 0 applies the policy in its fixed order and commits the caches and pending tokens.
 __device__ __forceinline__ void policy_commit(const PolicyArgs& A, int b, int lane, int last) {
+  // Everything the tail reads is requested before anything is used or stored (its stores may alias the loads as far as the
+  // compiler knows, and one trip to L2 after the other was most of this warp's time).
   const int a = A.n_accept[b];
-  long long r = 0;
+  const bool on = lane < A.n_dev;
+  long long* run_p = A.running + (long long)b * kMaxDev;
+  long long r = on ? run_p[lane] : 0;
+  const int head = A.h > 0 ? A.ring_head[b] : 0, count = A.h > 0 ? A.ring_count[b] : 0;
+  const long long pushed_old = A.pushed[b];
+  const int z = A.next_token[b], sib = A.sib_tok[b], y_last = A.tokens[b * A.G + A.G - 1], cnt = A.pending[b * 3];
+  const int len_old = A.kv_len && lane < A.m ? A.kv_len[b * A.m + lane] : 0;
   {
-    long long* run = A.running + (long long)b * kMaxDev;
-    const bool on = lane < A.n_dev;
-    if (on) r = run[lane];
-    int head = A.h > 0 ? A.ring_head[b] : 0, count = A.h > 0 ? A.ring_count[b] : 0;
-    for (int i = 0; i <= last; ++i) {
-      const long long dv = on ? __ldcg(A.dev + ((long long)b * A.G + i) * kMaxDev + lane) : 0;   // stored by this launch's clusters
-      if (A.h > 0) {
-        long long* slot = A.ring + ((long long)b * A.h + head) * kMaxDev;
-        const bool full = count == A.h;
-        if (on) {
-          if (full) r -= slot[lane];
-          slot[lane] = dv;
+    // position i enters the window; what leaves it is the ring's entry, or (window shorter than the block) position i - h
+    constexpr int kP = 8;                           // positions requested together
+    int at = head;
+#pragma unroll 1
+    for (int i0 = 0; i0 <= last; i0 += kP) {
+      long long dv[kP], old[kP];
+      const int at0 = at;
+#pragma unroll
+      for (int k = 0; k < kP; ++k) {
+        const int i = i0 + k;
+        dv[k] = 0; old[k] = 0;
+        if (i <= last && on) {
+          dv[k] = __ldcg(A.dev + ((long long)b * A.G + i) * kMaxDev + lane);               // stored by this launch's clusters
+          if (A.h > 0 && i < A.h && count + i >= A.h) old[k] = A.ring[((long long)b * A.h + at) * kMaxDev + lane];
         }
-        head = (head + 1) % A.h;
-        if (!full) count += 1;
+        if (++at >= A.h) at = 0;
       }
-      r += dv;
+#pragma unroll
+      for (int k = 0; k < kP; ++k) r += (A.h > 0 && i0 + k + A.h <= last ? 0 : dv[k]) - old[k];      // (or in and out again within the block)
+      if (A.h > 0) {
+        int w_at = at0;
+#pragma unroll
+        for (int k = 0; k < kP; ++k) {
+          if (i0 + k <= last && i0 + k + A.h > last && on) A.ring[((long long)b * A.h + w_at) * kMaxDev + lane] = dv[k];
+          if (++w_at >= A.h) w_at = 0;
+        }
+      }
     }
-    if (on) run[lane] = r;
-    if (lane == 0) {
-      if (A.h > 0) { A.ring_head[b] = head; A.ring_count[b] = count; }
-      A.pushed[b] += last + 1;
-    }
+    if (on) run_p[lane] = r;
+    if (A.h > 0 && lane == 0) { A.ring_head[b] = (head + last + 1) % A.h; A.ring_count[b] = min(A.h, count + last + 1); }
+    if (lane == 0) A.pushed[b] = pushed_old + last + 1;
   }
+  // commit: caches keep the pending token(s) and the accepted drafts that were fed
+  if (A.kv_len && lane < A.m) A.kv_len[b * A.m + lane] = len_old + cnt + (a < A.G ? a : A.G - 1);
   long long run[kMaxDev];
 #pragma unroll
   for (int kd = 0; kd < kMaxDev; ++kd) run[kd] = __shfl_sync(0xffffffffu, r, kd);
   if (lane != 0) return;
-  const long long pushed = A.pushed[b];
+  const long long pushed = pushed_old + last + 1;
 
   float* w = A.w + (long long)b * A.m;
   const float fx_scale = A.tvd ? 4.547473508864641e-13f : kMassInv;     // 2^-41 or 2^-40
@@ -973,7 +1004,7 @@ __device__ __forceinline__ void policy_commit(const PolicyArgs& A, int b, int la
     for (int k = 0; k < A.m; ++k) w[k] = s;
   } else if (A.policy == 5) {
     // AdaBoost-style weights from the drafters' error counts over the n window positions
-    const long long n = A.h > 0 ? (long long)A.ring_count[b] : pushed;
+    const long long n = A.h > 0 ? (long long)min(A.h, count + last + 1) : pushed;
     const float den = __fadd_rn(__ll2float_rn(n), 2.0f);
     const float lk = __fmul_rn(A.tau, xlog((float)(A.V - 1)));
     float t[8], tot = 0.0f;
@@ -1013,17 +1044,10 @@ __device__ __forceinline__ void policy_commit(const PolicyArgs& A, int b, int la
   if (A.out_w) for (int k = 0; k < A.m; ++k) A.out_w[(long long)b * A.m + k] = w[k];
   if (A.out_argmax) A.out_argmax[b] = am;
 
-  // commit: caches keep the pending token(s) and the accepted drafts that were fed
+  // what the target emitted beyond the caches is pending: the replacement; or an accepted sibling (token tree) or the last
+  // accepted draft of a fully accepted block, followed by the next token
   int* pend = A.pending + b * 3;
-  const int cnt = pend[0];
-  if (A.kv_len) {
-    const int keep = cnt + (a < A.G ? a : A.G - 1);
-    for (int k = 0; k < A.m; ++k) A.kv_len[b * A.m + k] += keep;
-  }
-  // ... and what the target emitted beyond them is pending: the replacement; or an accepted sibling (token tree) or the
-  // last accepted draft of a fully accepted block, followed by the next token
-  const int z = A.next_token[b], sib = A.sib_tok[b];
-  if (a == A.G) { pend[0] = 2; pend[1] = A.tokens[b * A.G + A.G - 1]; pend[2] = z; }
+  if (a == A.G) { pend[0] = 2; pend[1] = y_last; pend[2] = z; }
   else if (sib >= 0) { pend[0] = 2; pend[1] = sib; pend[2] = z; }
   else { pend[0] = 1; pend[1] = z; pend[2] = 0; }
 }
