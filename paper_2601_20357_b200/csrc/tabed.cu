@@ -74,7 +74,7 @@ struct tabed_handle {
   unsigned long long* chunk_mass = nullptr; ChunkBest* chunk_best = nullptr;
   int* err = nullptr;
   int cs_max = 8;                   // largest cluster the per-request kernels may use on this device (8 portable, 16 opt-in)
-  int cs_active[5] = {0, 0, 0, 0, 0};   // clusters of 1, 2, 4, 8, 16 CTAs that the device keeps resident at once
+  int cs_active[kReqMaxCluster + 1]{};  // clusters of so many CTAs that the device keeps resident at once
   bool req_dyn_ok = false;          // the cluster kernels may take up to kReqDynSmemMax of dynamic shared memory
   int cta_budget = 3;               // CTAs per SM a launch of the per-request kernels may have in total (3, 6, 12 measured: 3 best)
   // staging for the host-buffer entry point
@@ -197,6 +197,17 @@ int pick_cluster(const tabed_handle* h, int n_clusters, int* slice, int budget_s
   // (measured on 32 requests: many small CTAs in several waves beat one wave of large ones - the passes are bound by
   // dependent latencies and arithmetic, and more resident warps hide both)
   while (cs * 2 <= h->cs_max && (long long)n_clusters * cs * 2 <= (long long)h->cta_budget * budget_scale * n_sm && cs < by_v) cs *= 2;
+  *slice = ((h->V + cs - 1) / cs + 3) & ~3;
+  return cs;
+}
+
+// The ensemble step works every CTA for the whole launch, so a second wave costs a launch: the largest cluster, of any size,
+// with which all of them are resident.  (16 requests x 5 steps of 32000 tokens, a
+// whole round: 4 CTAs a cluster, two waves 156 us; 3 CTAs, one wave 148 us.)
+int pick_cluster_one_wave(const tabed_handle* h, int n_clusters, int* slice) {
+  const int by_v = (h->V + 1023) / 1024;
+  int cs = 1;
+  for (int c = 2; c <= std::min(h->cs_max, by_v); ++c) if (n_clusters <= h->cs_active[c]) cs = c;
   *slice = ((h->V + cs - 1) / cs + 3) & ~3;
   return cs;
 }
@@ -401,7 +412,7 @@ void run_ensemble(tabed_handle* h, const float* logits, const float* w, const fl
                   long long logits_step = 0) {
   ProfScope ps(h, TABED_PROF_ENSEMBLE);
   EnsembleArgs a{};
-  const int cs = pick_cluster(h, h->B * n_steps, &a.slice);
+  const int cs = pick_cluster_one_wave(h, h->B * n_steps, &a.slice);
   a.V = h->V; a.m = h->m; a.steps = n_steps; a.logits_step = logits_step; a.greedy = h->cfg.sample_mode == TABED_MODE_GREEDY;
   a.logits = logits; a.w = w; a.u = u; a.u_stride = u_stride;
   a.qk_out = qk_out; a.qk_req_stride = qk_stride; a.q_out = q_out; a.q_req_stride = q_stride;
@@ -977,18 +988,10 @@ int tabed_init(const tabed_config* cfg, const tabed_weights* wts, tabed_handle**
       for (const void* fn : {(const void*)k_ensemble_req, (const void*)k_verify_req, (const void*)k_verify_tail, (const void*)k_update_req})
         ok = ok && cudaOccupancyMaxActiveClusters(&n16, fn, &lc) == cudaSuccess && n16 >= 1;
       if (ok) h->cs_max = kReqMaxCluster;
-      // how many clusters of each size fit at once (the most demanding of the three kernels): a launch is sized for one wave
-      for (int i = 0; i < 5; ++i) {
-        const int cs = 1 << i;
-        if (cs > h->cs_max) break;
+      // how many clusters of each size fit at once (k_ensemble_req: a launch is sized for one wave)
+      for (int cs = 1; cs <= h->cs_max; ++cs) {
         lc.gridDim = dim3(cs); at[0].val.clusterDim.x = cs;
-        int best = 1 << 30;
-        for (const void* fn : {(const void*)k_ensemble_req, (const void*)k_verify_req, (const void*)k_verify_tail, (const void*)k_update_req}) {
-          int n = 0;
-          if (cudaOccupancyMaxActiveClusters(&n, fn, &lc) != cudaSuccess) n = 0;
-          best = std::min(best, n);
-        }
-        h->cs_active[i] = best;
+        if (cudaOccupancyMaxActiveClusters(&h->cs_active[cs], k_ensemble_req, &lc) != cudaSuccess) h->cs_active[cs] = 0;
       }
     }
     cudaGetLastError();
