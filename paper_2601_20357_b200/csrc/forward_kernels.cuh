@@ -175,7 +175,7 @@ constexpr int kGemvThreads = kGemvWarps * 32;
 template <typename T, int NS, int RPW, int EPI, bool ROUND_IN>
 __global__ void __launch_bounds__(kGemvThreads) k_gemv(GemvArgs A) {
   extern __shared__ __align__(16) float xs[];          // [NS][K]
-  __shared__ float red[kGemvWarps];
+  __shared__ float red[NS][kGemvWarps];
   constexpr int EL = Elem<T>::kPerVec;
   pdl_trigger();
   pdl_wait();
@@ -189,29 +189,48 @@ __global__ void __launch_bounds__(kGemvThreads) k_gemv(GemvArgs A) {
   }
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   // ---- prologue: stage (normalised, rounded) inputs ----
+  // All slots' rows and sums of squares in one trip and one block reduction (slot after slot they were 2 NS trips and 2 NS
+  // barriers, half of a small projection's time); the scaling then works on the thread's own staged elements.
+  const float* xin[NS];
+  float ss[NS];
+#pragma unroll
   for (int j = 0; j < NS; ++j) {
-    float* xj = xs + (long long)j * K;
-    if (j >= ns) { for (int i = tid; i < K; i += kGemvThreads) xj[i] = 0.0f; continue; }
-    const int src = A.src_slot ? A.src_slot[slot_base + j] : (slot_base + j);
-    const float* xin = A.in + (long long)src * A.in_stride;
-    float scale = 1.0f;
-    if (A.gain) {
-      float ss = 0.0f;
-      for (int i = tid; i < K; i += kGemvThreads) { const float v = xin[i]; ss = fmaf(v, v, ss); }
-      ss = warp_sum_f32(ss);
-      __syncthreads();
-      if (lane == 0) red[warp] = ss;
-      __syncthreads();
+    const int jj = min(j, ns - 1), src = A.src_slot ? A.src_slot[slot_base + jj] : (slot_base + jj);
+    xin[j] = A.in + (long long)src * A.in_stride;
+    ss[j] = 0.0f;
+  }
+  const T* g = reinterpret_cast<const T*>(A.gain);
+  for (int i = tid; i < K; i += kGemvThreads) {
+    float v[NS];
+#pragma unroll
+    for (int j = 0; j < NS; ++j) v[j] = j < ns ? xin[j][i] : 0.0f;
+#pragma unroll
+    for (int j = 0; j < NS; ++j) {
+      ss[j] = fmaf(v[j], v[j], ss[j]);
+      xs[(long long)j * K + i] = (!A.gain && ROUND_IN) ? Elem<T>::round(v[j]) : v[j];
+    }
+  }
+  if (A.gain) {
+#pragma unroll
+    for (int j = 0; j < NS; ++j) {
+      ss[j] = warp_sum_f32(ss[j]);
+      if (lane == 0) red[j][warp] = ss[j];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < NS; ++j) {
       float tot = 0.0f;
 #pragma unroll
-      for (int w = 0; w < kGemvWarps; ++w) tot += red[w];
-      scale = 1.0f / sqrtf(tot / (float)K + A.eps);
+      for (int w = 0; w < kGemvWarps; ++w) tot += red[j][w];
+      ss[j] = 1.0f / sqrtf(tot / (float)K + A.eps);
     }
-    const T* g = reinterpret_cast<const T*>(A.gain);
     for (int i = tid; i < K; i += kGemvThreads) {
-      float v = xin[i];
-      if (A.gain) v = v * scale * Elem<T>::load(g + i);
-      xj[i] = ROUND_IN ? Elem<T>::round(v) : v;
+      const float gi = Elem<T>::load(g + i);
+#pragma unroll
+      for (int j = 0; j < NS; ++j) {
+        const float v = xs[(long long)j * K + i] * ss[j] * gi;
+        xs[(long long)j * K + i] = ROUND_IN ? Elem<T>::round(v) : v;
+      }
     }
   }
   __syncthreads();
@@ -365,7 +384,7 @@ template <typename T, int HD>
 __global__ void __launch_bounds__(kAttnThreads)
 k_attn_partial(const float* __restrict__ qkv, const SlotDesc* __restrict__ slots, int H, int Hkv,
                const T* __restrict__ kc, const T* __restrict__ vc, int layer, int L, int cap, int split_len,
-               float* __restrict__ part_o, float* __restrict__ part_ml, int max_splits, float scale) {
+               float* __restrict__ part_o, float* __restrict__ part_ml, int max_splits, float scale, float* __restrict__ out) {
   constexpr int EL = Elem<T>::kPerVec;
   constexpr int LPR = HD / EL;                 // lanes per cache row
   constexpr int PPW = 32 / LPR;                // positions per warp pass
@@ -472,6 +491,7 @@ k_attn_partial(const float* __restrict__ qkv, const SlotDesc* __restrict__ slots
 #pragma unroll
       for (int w = 0; w < NW; ++w) v += s_o[w][t][dd];
       const int head = g * grp + t0 + t;
+      if (out) { out[((long long)s * H + head) * HD + dd] = v / s_l[t]; continue; }      // one split: nothing to merge
       const long long pi = ((long long)s * H + head) * max_splits + split;
       part_o[pi * HD + dd] = v;
       if (dd == 0) { part_ml[pi * 2] = s_m[t]; part_ml[pi * 2 + 1] = s_l[t]; }

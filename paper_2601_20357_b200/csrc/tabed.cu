@@ -338,8 +338,8 @@ void launch_attention_hd(tabed_handle* h, int layer, int n_slots, int max_pos, u
   auto merge = k_attn_merge<HD>;
   TABED_LAUNCH_PDL(h, part, dim3(splits, h->Hkv, n_slots), kAttnThreads, 0, h->qkv, h->slots, h->H, h->Hkv,
                reinterpret_cast<const T*>(h->kc), reinterpret_cast<const T*>(h->vc), layer, h->L, h->cap, split_len,
-               h->part_o, h->part_ml, h->max_splits, scale);
-  TABED_LAUNCH_PDL(h, merge, dim3(h->H, n_slots), HD, 0, h->slots, h->H, split_len, h->part_o, h->part_ml,
+               h->part_o, h->part_ml, h->max_splits, scale, splits == 1 && !act_out ? h->attn_out : (float*)nullptr);
+  if (splits > 1 || act_out) TABED_LAUNCH_PDL(h, merge, dim3(h->H, n_slots), HD, 0, h->slots, h->H, split_len, h->part_o, h->part_ml,
                h->max_splits, h->attn_out, act_out, act_npad, act_chunks);
 }
 
