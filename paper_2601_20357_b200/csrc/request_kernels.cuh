@@ -348,7 +348,7 @@ __global__ void __launch_bounds__(kReqThreads, 2) k_ensemble_req(const EnsembleA
   cg::cluster_group cluster = cg::this_cluster();
   __shared__ ReqShared S;
   const ReqCtx c = req_ctx(cluster, A.V, A.slice);
-  const int unit = blockIdx.x / c.CS, b = unit / A.steps, step = unit - b * A.steps, m = A.m, V = A.V;
+  const int unit = blockIdx.x / c.CS, b = A.steps == 1 ? unit : unit / A.steps, step = unit - b * A.steps, m = A.m, V = A.V;
   float* ebuf = A.ebuf_pitch > 0 ? reinterpret_cast<float*>(req_dyn_smem) : nullptr;
   const int epitch = A.ebuf_pitch;
   pdl_wait();
