@@ -1,6 +1,6 @@
 """The fused layer projections and the prompt attention at the sizes where their tiles end: a prompt fed in chunks through
 the tensor-core kernels, and a decoder step of many rows, against the same work one kernel per operation (each of the two is
-within the checker's bound, so they differ by at most twice that bound)."""
+within the bound that holds against the oracle, so they differ by at most twice that bound)."""
 import numpy as np
 import pytest
 import torch
