@@ -1,19 +1,16 @@
-// Weight-shared projections for MANY rows (batched serving: 32 requests x 3 inputs = 96 shared-weight
-// rows, 192 slots when every request feeds two pending tokens): out[slot][o] = sum_k W[o][k] act[slot][k]
-// on the 5th-generation tensor cores.  With ~100 rows per weight byte this is a real dense
-// contraction (the SIMT path re-reads the weights once per 8 rows), so it runs as tcgen05.mma with
-// the accumulator in tensor memory:
+// The plain tensor-core projection: out[slot][o] = sum_k W[o][k] act[slot][k] on the 5th-generation tensor cores, for the LM
+// head of the tensor-core path (the layers' projections, with everything around the product, are k_proj_tc) and for
+// tabed_debug_gemm_tc.
 //
 //   D[128 weight rows][N slots] += A[128][16] * B[N][16]^T     (kind::f16, bf16 inputs, fp32 accumulate)
 //
-// * A work unit is (tile of 128 weight rows, range of input columns); split-K over the input
-//   dimension gives >= one unit per SM even for the 768-row projections.  Units write fp32 partial
-//   sums [k-split][slot][row]; the consumer of the projection adds them in k-split order (deterministic).
+// * A work unit is (tile of 128 weight rows, range of input columns).  Units write fp32 partial sums
+//   [k-split][slot][row] (the LM head has one split: its logits are stored directly).
 // * Operands reach shared memory by bulk asynchronous copies (cp.async.bulk + mbarrier), three stages of
 //   128 input columns.  Both operands are stored in global memory already in the tensor core's canonical
 //   K-major, no-swizzle layout (8 rows x 16 bytes core matrices), so a stage is two contiguous copies and
 //   needs no tensor map: the weights are re-laid once at set-up (k_pack_tc), the activations by the kernel
-//   that normalises and rounds them (k_prep_act).
+//   that normalises and rounds them (k_prep_row).
 // * One thread issues the copies and the MMAs; tcgen05.commit releases a stage / signals the epilogue;
 //   eight warps read the accumulator with tcgen05.ld (warps w and w + 4 own TMEM lanes 32w..32w+31, half of the columns each) and store
 //   coalesced rows.  Every wait is bounded; on a timeout the CTA sets an error bit, drains and frees TMEM.
@@ -44,7 +41,6 @@ struct TcGemmArgs {
   const unsigned char* b_packed;   // [k_chunks] blocks of n_pad rows
   float* partial;                  // [ks] slabs of `slab` floats; slab layout [slot][rows_total], first slot of this launch at +0
   size_t slab;                     // floats between k-split slabs
-  const SlotDesc* slots;           // optional: the launch returns at once when none of its slots is active
   int rows_total;                  // output rows of the projection (multiple of 128 after padding in a_packed)
   int rows_valid;                  // rows actually stored
   int n_pad, n_slots;              // MMA N (multiple of 16) / slots stored
@@ -119,28 +115,6 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_gemm_tc(const TcGemmArgs G) {
     }
   }
   pdl_wait();
-  {
-    int any = 1;
-    if (G.slots) {
-      any = 0;
-      for (int s = tid; s < G.n_slots; s += kTcThreads) any |= G.slots[s].active;
-    }
-    if (!__syncthreads_or(any)) {
-      // nobody needs this pass: let the weight copies land, give the tensor memory back, leave
-      if (tid == 0) {
-        for (int c = 0; c < pre; ++c) {
-          mbar_expect_tx(&s_full[c], 0u);
-          unsigned spins = 0;
-          while (!mbar_try_wait(&s_full[c], 0) && ++spins < (1u << 20)) __nanosleep(32);
-        }
-      }
-      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      __syncthreads();
-      if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(tmem_cols) : "memory");
-      return;
-    }
-  }
-
   if (tid == 0 && n_ch > 0) {
     // instruction descriptor: fp32 accumulator, bf16 x bf16, both operands K-major, N and M
     const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(G.n_pad >> 3) << 17) | ((uint32_t)(kTcM >> 4) << 24);
