@@ -425,11 +425,12 @@ __global__ void __launch_bounds__(128) k_prep_row(const PrepRowArgs P) {
   if (P.slots && !P.slots[s].active) return;
   const float sc = proj_rms_scale(P.ss + (size_t)s * P.n_ss, P.n_ss, P.d, P.eps);
   const float* xr = P.x + (size_t)s * P.d;
-  for (int k = threadIdx.x * 8; k < P.d; k += 128 * 8) {
+  for (int k = threadIdx.x * 8; k < P.k_chunks * kTcKC; k += 128 * 8) {
+    uint4 v = make_uint4(0u, 0u, 0u, 0u);                      // (beyond d: tc_act_offset)
+    if (k >= P.d) { *reinterpret_cast<uint4*>(P.dst + tc_act_offset(r, k, P.n_pad, P.k_chunks)) = v; continue; }
     const float4 a = *reinterpret_cast<const float4*>(xr + k), b = *reinterpret_cast<const float4*>(xr + k + 4);
     float g[8];
     Elem<__nv_bfloat16>::unpack(__ldg(reinterpret_cast<const uint4*>(P.gain + k)), g);
-    uint4 v;
     v.x = pack_bf16(a.x * sc * g[0], a.y * sc * g[1]); v.y = pack_bf16(a.z * sc * g[2], a.w * sc * g[3]);
     v.z = pack_bf16(b.x * sc * g[4], b.y * sc * g[5]); v.w = pack_bf16(b.z * sc * g[6], b.w * sc * g[7]);
     *reinterpret_cast<uint4*>(P.dst + tc_act_offset(r, k, P.n_pad, P.k_chunks)) = v;

@@ -655,7 +655,7 @@ int setup_tc(tabed_handle* h) {
   auto A2 = [&](auto** ptr, size_t count, bool zero) { if (rc == TABED_OK) rc = dev_alloc(h, ptr, count, zero); };
   const size_t S2 = (size_t)h->slot_cap * 3 / 2 + kTcMaxN, n_ss = proj_n_ss(h);       // (tiles of at least 32 slots, padded to 16)
   A2(&h->tc_w, h->tc_off[KIND_LM] + h->tck[KIND_LM].bytes, false);
-  // (zeroed: columns beyond the operand's K and slots nobody wrote only meet zero weights or unused outputs, but must be finite)
+  // (slots that nobody writes only reach outputs that nobody reads; a slot's columns beyond the operand's K are its writer's)
   A2(&h->tc_act, S2 * std::max(h->tck[KIND_QKV].k_chunks, h->tck[KIND_O].k_chunks) * kTcKC * 2, true);
   A2(&h->tc_mid, S2 * h->tck[KIND_DN].k_chunks * kTcKC * 2, true);
   A2(&h->tc_ss_a, n_ss * h->slot_cap, true); A2(&h->tc_ss_m, n_ss * h->slot_cap, true);

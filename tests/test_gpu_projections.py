@@ -63,3 +63,31 @@ def test_rows_at_tile_edges_agree_with_per_operation_step(B, m):
     a = _logits_after(wl, weights, TB.PATH_TENSOR_CORE, lengths, 6)
     b = _logits_after(wl, weights, TB.PATH_PER_OP, lengths, 6)
     assert np.max(np.abs(a - b)) <= 2 * H.logit_tols(wl)[0]
+
+
+@pytest.mark.parametrize("path", [TB.PATH_AUTO, TB.PATH_TENSOR_CORE] if torch.cuda.is_available() else [])
+@pytest.mark.parametrize("heads,kv_heads,hd", [(5, 1, 64), (5, 5, 64), (10, 10, 32)])
+def test_a_request_that_is_not_finite_leaves_the_others_alone(heads, kv_heads, hd, path):
+    """320 columns end in the middle of an operand block.  What the blocks hold there must not come from another slot: the
+    prompts, the decoder step and its LM head cut the same buffer differently, so the values of a request whose embeddings
+    are NaN lie under every part of the layouts that follow.  The other request's logits keep their bits."""
+    wl = _workload(2, 3, heads, kv_heads, hd, 640, 400)
+    weights = TB.weights_to_device(wl.drafter, W.make_weights(wl), torch.device("cuda", 0))
+    gen = torch.Generator(device="cuda").manual_seed(9)
+    emb = [torch.randn((n, wl.drafter.d_model), generator=gen, device="cuda") for n in (37, 130, 5, 300, 64, 129)]
+    tok = torch.randint(0, wl.drafter.vocab, (2,), generator=gen, device="cuda", dtype=torch.int32)
+    seen = []
+    for bad in (False, True):
+        g = _handle(wl, weights)
+        g.select_path(path)
+        for row in (3, 0, 4, 1, 5, 2):
+            g.prefill_embeds(row, torch.full_like(emb[row], float("nan")) if bad and row >= 3 else emb[row])
+        out = torch.empty((2, wl.n_rows, wl.drafter.vocab), device="cuda")
+        for i in range(2):
+            g.decode_step(tok, out[i])
+        torch.cuda.synchronize()
+        seen.append(out[:, :3].cpu().numpy())
+        assert np.isfinite(seen[-1]).all()
+        assert not bad or not np.isfinite(out[:, 3:].cpu().numpy()).any()
+        g.destroy()
+    assert np.array_equal(seen[0], seen[1])
