@@ -35,8 +35,9 @@ struct PromptAttnArgs {
   unsigned char* act_out; int act_npad, act_chunks;      // the output as the next projection's operand blocks
 };
 
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+// 16 bytes, of which the first n (0 or 16) come from src and the rest are zero
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, uint32_t n) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(n) : "memory");
 }
 
 // grid (tiles of 16 QW positions, H)
@@ -53,7 +54,7 @@ __global__ void __launch_bounds__(QW * 32 * prompt_attn_groups<HD, QW>(), 1) k_p
   pdl_wait();
   const SlotDesc first = A.slots[0];
   const int q0 = (gridDim.x - 1 - blockIdx.x) * kPaQ, head = blockIdx.y, hk = head / (A.H / A.Hkv);
-  const int q_last = min(q0 + kPaQ, A.n) - 1, n_tiles = (first.pos + q_last) / kPaT + 1;
+  const int last = min(first.pos + min(q0 + kPaQ, A.n) - 1, A.cap - 1), n_tiles = last / kPaT + 1;      // last cache position needed
   const size_t base = ((((size_t)first.row * A.L + A.layer) * A.Hkv + hk) * A.cap) * HD;
   const __nv_bfloat16 *kb = A.kc + base, *vb = A.vc + base;
   constexpr uint32_t TILE = kPaT * HD * 2;
@@ -65,9 +66,12 @@ __global__ void __launch_bounds__(QW * 32 * prompt_attn_groups<HD, QW>(), 1) k_p
 #pragma unroll 4
     for (int i = tid; i < kPaT * PIECES; i += kPaGroup) {
       const int r = i / PIECES, c = i - r * PIECES;
-      const int p = min(t * kPaT + r, A.cap - 1);             // (rows past the last position are masked, but stay inside the cache)
-      cp_async16(kd + piece(r, c), kb + (size_t)p * HD + c * 8);
-      cp_async16(vd + piece(r, c), vb + (size_t)p * HD + c * 8);
+      // rows past the last position are masked, but a weight of 0 does not cancel what an earlier, longer prompt of the row
+      // may have left there if that is not finite: they read as zeros
+      const int p = min(t * kPaT + r, last);
+      const uint32_t n = t * kPaT + r <= last ? 16u : 0u;
+      cp_async16(kd + piece(r, c), kb + (size_t)p * HD + c * 8, n);
+      cp_async16(vd + piece(r, c), vb + (size_t)p * HD + c * 8, n);
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
   };

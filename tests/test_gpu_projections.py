@@ -91,3 +91,30 @@ def test_a_request_that_is_not_finite_leaves_the_others_alone(heads, kv_heads, h
         assert not bad or not np.isfinite(out[:, 3:].cpu().numpy()).any()
         g.destroy()
     assert np.array_equal(seen[0], seen[1])
+
+
+@pytest.mark.parametrize("heads,kv_heads,hd", [(8, 4, 32), (2, 1, 128)])
+def test_a_prompt_does_not_see_what_a_longer_one_left_in_the_cache(heads, kv_heads, hd):
+    """The cache beyond a prompt's last position may still hold an earlier conversation of the row, and that need not have
+    been finite: after the saved state is restored, the logits of a shorter prompt have the bits of a fresh handle."""
+    wl = _workload(1, 3, heads, kv_heads, hd, 640, 200)
+    weights = TB.weights_to_device(wl.drafter, W.make_weights(wl), torch.device("cuda", 0))
+    gen = torch.Generator(device="cuda").manual_seed(10)
+    emb = [torch.randn((n, wl.drafter.d_model), generator=gen, device="cuda") for n in (17, 65, 100)]
+    tok = torch.randint(0, wl.drafter.vocab, (1,), generator=gen, device="cuda", dtype=torch.int32)
+    seen = []
+    for used in (False, True):
+        g = _handle(wl, weights)
+        saved = g.state_export()
+        if used:
+            for row in range(3):
+                g.prefill_embeds(row, torch.full((190, wl.drafter.d_model), float("nan"), device="cuda"))
+            g.state_import(saved)
+        for row in range(3):
+            g.prefill_embeds(row, emb[row])
+        out = torch.empty((wl.n_rows, wl.drafter.vocab), device="cuda")
+        g.decode_step(tok, out)
+        torch.cuda.synchronize()
+        seen.append(out.cpu().numpy())
+        g.destroy()
+    assert np.isfinite(seen[1]).all() and np.array_equal(seen[0], seen[1])
