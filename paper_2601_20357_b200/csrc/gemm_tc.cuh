@@ -19,22 +19,16 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "proj_plan.h"
 #include "round_kernel.cuh"   // PTX wrappers: mbarrier, bulk copy
 
 namespace tabed {
 
-constexpr int kTcM = 128;          // weight rows per tile (MMA M)
-constexpr int kTcKC = 128;         // input columns per pipeline stage
 constexpr int kTcStages = 3;        // pipeline stages (2 when more than 128 slots share the shared memory)
 constexpr int kTcMaxStages = 8;
 constexpr int kTcThreads = 256;      // eight warps: warps w and w + 4 read the same 32 accumulator lanes, half of the columns each
 constexpr int kPrefillChunk = 1024;       // positions of one row prefilled as slots of one weight pass
-constexpr int kTcMaxN = 256;       // slots per launch (MMA N is their count rounded up to 16)
 __host__ __device__ inline int tc_stages(int n_pad) { return n_pad > 128 ? 2 : kTcStages; }
-
-// Canonical K-major no-swizzle operand block of `rows` rows x kTcKC columns (bf16):
-// element (r, k) at ((k/8) * (rows/8) + r/8) * 128 + (r%8) * 16 + (k%8) * 2 bytes.
-__host__ __device__ inline size_t tc_block_bytes(int rows) { return (size_t)rows * kTcKC * 2; }
 
 struct TcGemmArgs {
   const unsigned char* a_packed;   // [m_tiles][k_chunks] blocks of 128 rows
@@ -82,7 +76,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_gemm_tc(const TcGemmArgs G) {
   const int c_lo = split * G.cps, c_hi = min(c_lo + G.cps, G.k_chunks), n_ch = (c_hi - c_lo) * per_chunk;
   const size_t a_bytes = tc_block_bytes(kTcM) / per_chunk, b_bytes = tc_block_bytes(G.n_pad) / per_chunk;
   const int n_stages = G.n_stages;
-  const uint32_t tmem_cols = G.n_pad <= 32 ? 32u : (G.n_pad <= 64 ? 64u : (G.n_pad <= 128 ? 128u : 256u));
+  const uint32_t tmem_cols = (uint32_t)tc_tmem_cols(G.n_pad);
 
   if (tid == 0) {
     for (int s = 0; s < n_stages; ++s) { mbar_init(&s_full[s], 1); mbar_init(&s_empty[s], 1); }

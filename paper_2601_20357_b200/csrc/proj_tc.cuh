@@ -28,11 +28,6 @@
 
 namespace tabed {
 
-constexpr int kProjMaxSplit = 8;      // CTAs of a cluster (portable size)
-constexpr int kProjMaxStages = 8;
-constexpr size_t kProjHalfSmem = 112u * 1024u;     // dynamic shared memory of a CTA that leaves room for a second one on its SM
-constexpr size_t kProjMaxSmem = 220u * 1024u;      // ... of one that has the SM to itself
-
 enum ProjEpi { PROJ_QKV = 0, PROJ_RESID = 1, PROJ_SWIGLU = 2 };
 
 struct ProjArgs {
@@ -57,12 +52,6 @@ struct ProjArgs {
   unsigned char* act_out; int act_npad, act_chunks;       // SWIGLU: operand blocks of the down projection (its tiles, its k_chunks)
   int* err;
 };
-
-// Bytes of one 128-column block of the operand that the RMSNorm prologue builds: its 8-column groups are 16 bytes further
-// apart than in a packed block, so that a warp's stores of one slot (16 groups) fall into different banks.
-__host__ __device__ inline unsigned proj_norm_block_bytes(int n_pad) { return 16u * ((unsigned)n_pad * 16u + 16u); }
-// Slots that one CTA of the cluster finishes: they are dealt round-robin.
-__host__ __device__ inline int proj_owned(int n_pad, int ks) { return (n_pad + ks - 1) / ks; }
 
 __device__ __forceinline__ float proj_rms_scale(const float* __restrict__ ss_row, int n_ss, int d, float eps) {
   float ss = 0.0f;
@@ -94,7 +83,7 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_proj_tc(const ProjArgs P) {
   const int c_lo = split * P.cps, c_hi = min(c_lo + P.cps, P.k_chunks), n_ch = c_hi - c_lo;   // (the host leaves no split empty)
   const int n_stages = P.n_stages;
   const unsigned a_bytes = (unsigned)tc_block_bytes(kTcM), b_bytes = P.x ? proj_norm_block_bytes(P.n_pad) : (unsigned)tc_block_bytes(P.n_pad);
-  const uint32_t tmem_cols = P.n_pad <= 32 ? 32u : (P.n_pad <= 64 ? 64u : (P.n_pad <= 128 ? 128u : 256u));
+  const uint32_t tmem_cols = (uint32_t)tc_tmem_cols(P.n_pad);
   unsigned char* a_ring = pj_smem;
   unsigned char* b_area = pj_smem + (size_t)n_stages * a_bytes;
   const bool push = P.recv_off != 0;

@@ -43,9 +43,6 @@ struct DeviceGuard {
 
 }  // namespace
 
-// A layer projection's cut into slot tiles and K splits (plan_proj).
-struct ProjPlan { int n_pad, n_tiles, ks, cps, n_stages; bool norm; unsigned recv_off; size_t smem; float us; };
-
 struct tabed_handle {
   tabed_config cfg;
   bool has_drafter = false;
@@ -694,63 +691,15 @@ void launch_lm_head_tc(tabed_handle* h, const unsigned char* act, int n, int n_p
   TABED_LAUNCH_PDL(h, k_gemm_tc, t.m_tiles, kTcThreads, smem, G);
 }
 
-// How a layer projection over n_slots slots is cut into slot tiles and K splits.  What a choice costs, in us, as measured on
-// the kernel's own time line (18 - 1024 slots, 768 - 4864 columns): a CTA draws 75 KB/us alone and all of them together
-// 6.5 MB/us from L2; 8 slots of the epilogue cost each warp 0.2 us; the exchange between the CTAs of a cluster 1 us, and
-// 0.02 us per slot more where the slabs are pulled for lack of a receive buffer; a normalising prologue 1.2 us and 0.02 us per
-// slot and 128 columns, against 3 us for a launch that packs the operand; a wave that is not full costs a wave.
-ProjPlan plan_proj(const tabed_handle* h, int kind, int n_slots, bool can_norm) {
-  const tabed_handle::TcKind& t = h->tck[kind];
-  ProjPlan best{};
-  best.us = 1e30f;
-  int last_pad = 0;
-  for (int tiles = (n_slots + kTcMaxN - 1) / kTcMaxN; tiles <= std::max(1, n_slots / 32); ++tiles) {
-    const int n_pad = ((n_slots + tiles - 1) / tiles + 15) / 16 * 16;
-    if (n_pad == last_pad) continue;
-    last_pad = n_pad;
-    const int n_tiles = (n_slots + n_pad - 1) / n_pad, units = t.m_tiles * n_tiles;
-    const size_t a = tc_block_bytes(kTcM), b = tc_block_bytes(n_pad), bn = proj_norm_block_bytes(n_pad), slab = (size_t)n_pad * kTcM * sizeof(float);
-    for (int want = 1; want <= std::min(kProjMaxSplit, t.k_chunks); ++want) {
-      const int cps = (t.k_chunks + want - 1) / want, ks = (t.k_chunks + cps - 1) / cps;
-      if (ks != want) continue;
-      const size_t recv = ks > 1 ? (size_t)ks * proj_owned(n_pad, ks) * kTcM * sizeof(float) : 0;
-      const int deep = std::min(cps, kProjMaxStages), least = std::min(2, deep);
-      for (int norm = 0; norm <= (can_norm ? 1 : 0); ++norm) {
-        const size_t fixed = norm ? (size_t)cps * bn : 0, per_stage = norm ? a : a + b;
-        for (int half = 0; half < 2; ++half) {
-          const size_t budget = half ? kProjHalfSmem : kProjMaxSmem;
-          // slabs are pushed where the receive buffer fits beside the operands, else pulled
-          const size_t extra = recv && fixed + recv + least * per_stage <= budget ? recv : 0;
-          if (std::max(fixed + extra + least * per_stage, extra ? 0 : slab) > budget) continue;
-          ProjPlan p{};
-          p.n_pad = n_pad; p.n_tiles = n_tiles; p.ks = ks; p.cps = cps; p.norm = norm != 0;
-          p.n_stages = (int)std::min<size_t>(deep, (budget - fixed - extra) / per_stage);
-          const size_t operands = fixed + p.n_stages * per_stage;
-          p.recv_off = extra ? (unsigned)operands : 0u;
-          p.smem = std::max(operands + extra, extra ? 0 : slab);
-          const int fit = std::max(1, h->proj_fit[ks] * (p.smem <= kProjHalfSmem ? 2 : 1)) * ks, ctas = units * ks;
-          const float waves = (float)((ctas + fit - 1) / fit);
-          const float rate = std::min(p.n_stages >= std::min(deep, 3) ? 75.0f : 60.0f, 6500.0f / (float)std::min(ctas, fit));       // KB per us and CTA
-          p.us = waves * ((float)(cps * (a + b)) / 1024.0f / rate + 2.0f + 0.25f * (float)((proj_owned(n_pad, ks) + 7) / 8) + (ks > 1 ? 1.0f : 0.0f) +
-                          (ks > 1 && !extra ? 0.02f * (float)n_pad : 0.0f) + (norm ? 1.2f + 0.02f * (float)(std::min(n_pad, n_slots) * cps) : 0.0f)) +
-                 (can_norm && !norm ? 3.0f : 0.0f) - (p.smem <= kProjHalfSmem ? 0.5f : 0.0f);      // (room for the next kernel's start)
-          if (p.us < best.us) best = p;
-        }
-      }
-    }
-  }
-  return best;                                                 // (256 slots in one CTA: two stages are 192 KB - always found)
-}
-
 // The plans of a step, kept for the few slot counts that a handle's steps have in turn (2 R and R; a prompt's chunks).
 const tabed_handle::StepPlan& step_plan(tabed_handle* h, int n_slots) {
   for (const auto& e : h->step_plans) if (e.n_slots == n_slots) return e;
   tabed_handle::StepPlan e;
   e.n_slots = n_slots;
-  e.p[KIND_QKV] = plan_proj(h, KIND_QKV, n_slots, true);
-  e.p[KIND_O] = plan_proj(h, KIND_O, n_slots, false);
-  e.p[KIND_GU] = plan_proj(h, KIND_GU, n_slots, true);
-  e.p[KIND_DN] = plan_proj(h, KIND_DN, n_slots, false);
+  e.p[KIND_QKV] = plan_proj(h->tck[KIND_QKV].m_tiles, h->tck[KIND_QKV].k_chunks, n_slots, true, h->proj_fit);
+  e.p[KIND_O] = plan_proj(h->tck[KIND_O].m_tiles, h->tck[KIND_O].k_chunks, n_slots, false, h->proj_fit);
+  e.p[KIND_GU] = plan_proj(h->tck[KIND_GU].m_tiles, h->tck[KIND_GU].k_chunks, n_slots, true, h->proj_fit);
+  e.p[KIND_DN] = plan_proj(h->tck[KIND_DN].m_tiles, h->tck[KIND_DN].k_chunks, n_slots, false, h->proj_fit);
   if (h->step_plans.size() >= 16) h->step_plans.erase(h->step_plans.begin());
   h->step_plans.push_back(e);
   return h->step_plans.back();
