@@ -118,7 +118,8 @@ struct tabed_handle {
                                                         // layer and between its attention and its MLP
   size_t tc_smem = 0;
   struct StepPlan { int n_slots; ProjPlan p[4]; };
-  std::vector<StepPlan> step_plans;
+  StepPlan step_plans[16]{};        // (n_slots 0: none yet)
+  int next_plan = 0;
   int proj_fit[9]{};                // resident clusters of 1 .. 8 CTAs of a projection, one CTA per SM
   // per-kernel-class timing (tabed_profile_begin / tabed_profile_end)
   int prof_class = -1;
@@ -691,18 +692,18 @@ void launch_lm_head_tc(tabed_handle* h, const unsigned char* act, int n, int n_p
   TABED_LAUNCH_PDL(h, k_gemm_tc, t.m_tiles, kTcThreads, smem, G);
 }
 
-// The plans of a step, kept for the few slot counts that a handle's steps have in turn (2 R and R; a prompt's chunks).
+// The plans of a step, kept for the few slot counts that a handle's steps have in turn (2 R and R; a prompt's chunks) in a
+// fixed table: nothing on the way of a call allocates, and nothing can throw through the C boundary.
 const tabed_handle::StepPlan& step_plan(tabed_handle* h, int n_slots) {
   for (const auto& e : h->step_plans) if (e.n_slots == n_slots) return e;
-  tabed_handle::StepPlan e;
+  tabed_handle::StepPlan& e = h->step_plans[h->next_plan];
+  h->next_plan = (h->next_plan + 1) % 16;
   e.n_slots = n_slots;
   e.p[KIND_QKV] = plan_proj(h->tck[KIND_QKV].m_tiles, h->tck[KIND_QKV].k_chunks, n_slots, true, h->proj_fit);
   e.p[KIND_O] = plan_proj(h->tck[KIND_O].m_tiles, h->tck[KIND_O].k_chunks, n_slots, false, h->proj_fit);
   e.p[KIND_GU] = plan_proj(h->tck[KIND_GU].m_tiles, h->tck[KIND_GU].k_chunks, n_slots, true, h->proj_fit);
   e.p[KIND_DN] = plan_proj(h->tck[KIND_DN].m_tiles, h->tck[KIND_DN].k_chunks, n_slots, false, h->proj_fit);
-  if (h->step_plans.size() >= 16) h->step_plans.erase(h->step_plans.begin());
-  h->step_plans.push_back(e);
-  return h->step_plans.back();
+  return e;
 }
 
 template <int EPI>

@@ -118,3 +118,25 @@ def test_a_prompt_does_not_see_what_a_longer_one_left_in_the_cache(heads, kv_hea
         seen.append(out.cpu().numpy())
         g.destroy()
     assert np.isfinite(seen[1]).all() and np.array_equal(seen[0], seen[1])
+
+
+def test_more_slot_counts_than_the_table_of_plans_holds():
+    """A prompt fed in 22 pieces of 20 different lengths (the table has 16 places), against one position at a time."""
+    wl = _workload(1, 1, 4, 2, 64, 640, 240)
+    weights = TB.weights_to_device(wl.drafter, W.make_weights(wl), torch.device("cuda", 0))
+    gen = torch.Generator(device="cuda").manual_seed(11)
+    tok = torch.randint(0, wl.drafter.vocab, (214,), generator=gen, device="cuda", dtype=torch.int32)
+    seen = []
+    for path in (TB.PATH_TENSOR_CORE, TB.PATH_PER_OP):
+        g = _handle(wl, weights)
+        g.select_path(path)
+        at = 0
+        for n in (*range(1, 21), 1, 2):
+            g.prefill_tokens(0, tok[at:at + n].contiguous())
+            at += n
+        out = torch.empty((1, wl.drafter.vocab), device="cuda")
+        g.decode_step(tok[at:at + 1].contiguous(), out)
+        torch.cuda.synchronize()
+        seen.append(out.cpu().numpy())
+        g.destroy()
+    assert np.max(np.abs(seen[0] - seen[1])) <= 2 * H.logit_tols(wl)[0]
