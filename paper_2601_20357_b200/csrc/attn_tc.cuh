@@ -50,7 +50,6 @@ constexpr int kAtcTile = kAtcSplit * kAtcHd * 2;   // bytes of one K (or V) tile
 constexpr int kAtcMaxStages = 8;
 constexpr int kAtcMaxCtas = 1024;
 constexpr int kAtcMaxSlots = 512;
-constexpr int kAtcMaxCap = 1 << 20;          // positions of a row that fit the packed slot table
 constexpr unsigned kAtcMaxDynSmem = 220u * 1024u;   // dynamic shared memory of a CTA that has the SM to itself (static: ~3 KB)
 
 struct AttnTcArgs {
@@ -63,6 +62,9 @@ struct AttnTcArgs {
   float* out;                                // [n_slots][H][hd]; unused when act_out is given
   unsigned char* act_out;                    // or null: the output as the bf16 B operand of the next projection
   int act_npad, act_chunks;                  //   (tc_act_offset: tiles of act_npad slots, act_chunks blocks each; K = H * hd)
+  // row and position of a slot in one word: cap has pos_bits bits, and R 2^pos_bits <= 2 R cap < 2^32 (the caches' rows, R L Hkv
+  // cap of them, are counted in 31 bits by their tensor maps)
+  int pos_bits;
   float scale;
   int* err;
   int n_stages;
@@ -112,7 +114,7 @@ k_attn_tc_bf16(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
   __shared__ uint64_t empty[kAtcMaxStages];     // a stage's tiles have been read by all eight warps
   __shared__ int s_seg[kAtcMaxStages + 1];      // warps that have finished a segment (ring of n_stages + 1 segments)
   __shared__ int s_pref[kAtcMaxSlots + 1];
-  __shared__ unsigned s_rp[kAtcMaxSlots];       // (row << 20) | position: every slot is read from global memory once
+  __shared__ unsigned s_rp[kAtcMaxSlots];       // (row << pos_bits) | position: every slot is read from global memory once
   __shared__ int s_start;
   if (tid == 0) {
     for (int i = 0; i < n_stages; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], NW); }
@@ -123,7 +125,7 @@ k_attn_tc_bf16(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
   // chunks before every slot (prefix sums), built by the whole CTA
   for (int i = tid; i < n_slots; i += kAtcThreads) {
     const int4 sd = *reinterpret_cast<const int4*>(slots + i);                // row, pos, active
-    s_rp[i] = ((unsigned)sd.x << 20) | (unsigned)sd.y;
+    s_rp[i] = ((unsigned)sd.x << A.pos_bits) | (unsigned)sd.y;
     s_pref[i + 1] = sd.z ? Hkv * ((sd.y + SPLIT) / SPLIT) : 0;
   }
   __syncthreads();
@@ -149,6 +151,7 @@ k_attn_tc_bf16(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
   };
   for (int i = tid; i < n_slots; i += kAtcThreads)
     if (s_pref[i] <= g_lo && g_lo < s_pref[i + 1]) s_start = i;
+  const unsigned pos_mask = (1u << A.pos_bits) - 1u;
   struct Walk { int s, gk, split, nsplit, row, pos; };
   auto advance = [&](Walk& w) {                      // to the next chunk in (slot, head, position) order
     w.split++;
@@ -157,7 +160,7 @@ k_attn_tc_bf16(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
       if (w.gk == Hkv) {
         w.gk = 0;
         do { w.s++; } while (w.s < n_slots && s_pref[w.s + 1] == s_pref[w.s]);      // (inactive slots have no chunks)
-        if (w.s < n_slots) { w.row = (int)(s_rp[w.s] >> 20); w.pos = (int)(s_rp[w.s] & 0xFFFFFu); }
+        if (w.s < n_slots) { w.row = (int)(s_rp[w.s] >> A.pos_bits); w.pos = (int)(s_rp[w.s] & pos_mask); }
         w.nsplit = (w.pos + SPLIT) / SPLIT;
       }
     }
@@ -165,7 +168,7 @@ k_attn_tc_bf16(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
   auto seek = [&](int g, Walk& w) {                 // the (slot, head, split) of global chunk g < T
     int lo = 0, hi = n_slots;
     while (hi - lo > 1) { const int mid = (lo + hi) >> 1; if (s_pref[mid] <= g) lo = mid; else hi = mid; }
-    w.s = lo; w.row = (int)(s_rp[lo] >> 20); w.pos = (int)(s_rp[lo] & 0xFFFFFu);
+    w.s = lo; w.row = (int)(s_rp[lo] >> A.pos_bits); w.pos = (int)(s_rp[lo] & pos_mask);
     w.nsplit = (w.pos + SPLIT) / SPLIT;
     const int rem = g - s_pref[lo];
     w.gk = rem / w.nsplit; w.split = rem - w.gk * w.nsplit;
@@ -198,7 +201,7 @@ k_attn_tc_bf16(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
   if (g_lo < g_hi) {
     const int rem = g_lo - s_pref[s_start];
     cur.s = s_start;
-    cur.row = (int)(s_rp[s_start] >> 20); cur.pos = (int)(s_rp[s_start] & 0xFFFFFu);
+    cur.row = (int)(s_rp[s_start] >> A.pos_bits); cur.pos = (int)(s_rp[s_start] & pos_mask);
     cur.nsplit = (cur.pos + SPLIT) / SPLIT;
     cur.gk = rem / cur.nsplit;
     cur.split = rem - cur.gk * cur.nsplit;

@@ -309,10 +309,11 @@ void launch_attention_hd(tabed_handle* h, int layer, int n_slots, int max_pos, u
           const size_t smem2 = 1024 + n_stages * per_stage + seg_state;       // one more set of states than stages
           static bool attr2_set[kMaxDevices] = {false};
           if (!attr2_set[h->cfg.device]) { cudaFuncSetAttribute(k_attn_tc_bf16, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kAtcMaxDynSmem); attr2_set[h->cfg.device] = true; }
-          AttnTcArgs a;
+          AttnTcArgs a{};
           a.qkv = h->qkv; a.slots = h->slots; a.n_slots = n_slots; a.H = h->H; a.Hkv = h->Hkv; a.layer = layer; a.L = h->L;
           a.cap = h->cap; a.qkv_w = h->qkv_w; a.part_o = h->part_o; a.part_ml = h->part_ml; a.max_splits = h->max_splits;
           a.act_out = act_out; a.act_npad = act_npad; a.act_chunks = act_chunks;
+          while ((h->cap >> a.pos_bits) != 0) ++a.pos_bits;
           a.tickets = h->attn_tickets; a.out = h->attn_out; a.scale = 1.0f / sqrtf((float)h->hd); a.err = h->err; a.n_stages = n_stages;
           TABED_LAUNCH_PDL(h, k_attn_tc_bf16, n_ctas, kAtcThreads, smem2, h->tm_k, h->tm_v, a);
           return;
@@ -1006,7 +1007,7 @@ int tabed_init(const tabed_config* cfg, const tabed_weights* wts, tabed_handle**
       cudaDriverEntryPointQueryResult qres;
       const unsigned long long n_rows = (unsigned long long)R * h->L * h->Hkv * (unsigned long long)h->cap;
       if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &qres) == cudaSuccess && fn &&
-          qres == cudaDriverEntryPointSuccess && n_rows < (1ull << 31) && h->cap <= kAtcMaxCap) {
+          qres == cudaDriverEntryPointSuccess && n_rows < (1ull << 31)) {
         const cuuint64_t dims[2] = {(cuuint64_t)kAtcHd, (cuuint64_t)n_rows};
         const cuuint64_t strides[1] = {(cuuint64_t)kAtcHd * 2};
         const cuuint32_t box[2] = {(cuuint32_t)kAtcHd, (cuuint32_t)kAtcSplit};

@@ -1,6 +1,8 @@
 """The fused layer projections and the prompt attention at the sizes where their tiles end: a prompt fed in chunks through
 the tensor-core kernels, and a decoder step of many rows, against the same work one kernel per operation (each of the two is
 within the bound that holds against the oracle, so they differ by at most twice that bound)."""
+import dataclasses
+
 import numpy as np
 import pytest
 import torch
@@ -140,3 +142,22 @@ def test_more_slot_counts_than_the_table_of_plans_holds():
         seen.append(out.cpu().numpy())
         g.destroy()
     assert np.max(np.abs(seen[0] - seen[1])) <= 2 * H.logit_tols(wl)[0]
+
+
+def test_attention_of_a_capacity_beyond_2_to_the_20_takes_the_same_kernel():
+    """Row and position of a slot share a word in the attention kernel; more than 2^20 positions fit too."""
+    seen = []
+    for cap in (300, (1 << 20) + 9):
+        wl = _workload(1, 3, 2, 1, 64, 256, cap)
+        wl = dataclasses.replace(wl, drafter=dataclasses.replace(wl.drafter, n_layers=1))
+        weights = TB.weights_to_device(wl.drafter, W.make_weights(wl), torch.device("cuda", 0))
+        g = _handle(wl, weights)
+        gen = torch.Generator(device="cuda").manual_seed(12)
+        for row, n in enumerate((1, 127, 260)):
+            g.prefill_tokens(row, torch.randint(0, wl.drafter.vocab, (n,), generator=gen, device="cuda", dtype=torch.int32))
+        before, out = g.launch_count(), torch.empty((wl.n_rows, wl.drafter.vocab), device="cuda")
+        g.decode_step(torch.tensor([5], dtype=torch.int32, device="cuda"), out)
+        torch.cuda.synchronize()
+        seen.append((g.launch_count() - before, out.cpu().numpy()))
+        g.destroy()
+    assert seen[0][0] == seen[1][0] and np.array_equal(seen[0][1], seen[1][1])
