@@ -29,6 +29,9 @@ constexpr int kTcMaxStages = 8;
 constexpr int kTcThreads = 256;      // eight warps: warps w and w + 4 read the same 32 accumulator lanes, half of the columns each
 constexpr int kPrefillChunk = 1024;       // positions of one row prefilled as slots of one weight pass
 __host__ __device__ inline int tc_stages(int n_pad) { return n_pad > 128 ? 2 : kTcStages; }
+// The most dynamic shared memory that any launch takes (three stages of 128 slots, or two of 256).  The limit belongs to the
+// function, not to a launch: whoever sets it sets this value.
+constexpr size_t kTcMaxSmem = 3u * (kTcM + 128u) * kTcKC * 2u + 1024u;
 
 struct TcGemmArgs {
   const unsigned char* a_packed;   // [m_tiles][k_chunks] blocks of 128 rows

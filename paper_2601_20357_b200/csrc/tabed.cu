@@ -116,7 +116,6 @@ struct tabed_handle {
   unsigned char *tc_act = nullptr, *tc_mid = nullptr;   // operand blocks: normalised rows or attention outputs; gated products
   float *tc_ss_a = nullptr, *tc_ss_m = nullptr;         // partial sums of squares of the residual [slot][n_ss], entering a
                                                         // layer and between its attention and its MLP
-  size_t tc_smem = 0;
   struct StepPlan { int n_slots; ProjPlan p[4]; };
   StepPlan step_plans[16]{};        // (n_slots 0: none yet)
   int next_plan = 0;
@@ -626,13 +625,9 @@ int setup_tc(tabed_handle* h) {
   h->tc_off[KIND_DN] = h->tc_off[KIND_GU] + h->tck[KIND_GU].bytes;
   h->tc_layer_stride = h->tc_off[KIND_DN] + h->tck[KIND_DN].bytes;
   h->tc_off[KIND_LM] = h->tc_layer_stride * h->L;
-  const int n_pad_max = (std::min(h->slot_cap, kTcMaxN) + 15) / 16 * 16;
-  h->tc_smem = 0;
-  for (int np = 16; np <= n_pad_max; np += 16)
-    h->tc_smem = std::max(h->tc_smem, (size_t)tc_stages(np) * (tc_block_bytes(kTcM) + tc_block_bytes(np)) + 1024);
-  if (std::max(h->tc_smem, kProjMaxSmem) > (size_t)prop.sharedMemPerBlockOptin) return TABED_OK;
+  if (std::max(kTcMaxSmem, kProjMaxSmem) > (size_t)prop.sharedMemPerBlockOptin) return TABED_OK;
   auto smem_attr = [](auto kern, size_t bytes) { return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess; };
-  if (!smem_attr(k_gemm_tc, h->tc_smem) || !smem_attr(k_proj_tc<PROJ_QKV>, kProjMaxSmem) || !smem_attr(k_proj_tc<PROJ_RESID>, kProjMaxSmem) ||
+  if (!smem_attr(k_gemm_tc, kTcMaxSmem) || !smem_attr(k_proj_tc<PROJ_QKV>, kProjMaxSmem) || !smem_attr(k_proj_tc<PROJ_RESID>, kProjMaxSmem) ||
       !smem_attr(k_proj_tc<PROJ_SWIGLU>, kProjMaxSmem) || !smem_attr(k_prompt_attn<32, 4, 64>, prompt_attn_smem<32, 4, 64>()) ||
       !smem_attr(k_prompt_attn<64, 4, 64>, prompt_attn_smem<64, 4, 64>()) || !smem_attr(k_prompt_attn<128, 4, 64>, prompt_attn_smem<128, 4, 64>()) ||
       !smem_attr(k_prompt_attn<32, 2, 32>, prompt_attn_smem<32, 2, 32>()) || !smem_attr(k_prompt_attn<64, 2, 32>, prompt_attn_smem<64, 2, 32>()) ||
@@ -1644,7 +1639,7 @@ int tabed_debug_gemm_tc(const void* w, const float* act, int32_t rows, int32_t K
       cudaMalloc(&b_p, (size_t)k_chunks * tc_block_bytes(n_pad)) != cudaSuccess ||
       cudaMalloc(&part, (size_t)ks * n * rows * sizeof(float)) != cudaSuccess || cudaMalloc(&err, sizeof(int)) != cudaSuccess ||
       cudaMemsetAsync(err, 0, sizeof(int), st) != cudaSuccess ||
-      cudaFuncSetAttribute(k_gemm_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+      cudaFuncSetAttribute(k_gemm_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcMaxSmem) != cudaSuccess)
     rc = TABED_ERR_CUDA;
   if (rc == TABED_OK) {
     k_pack_tc<<<dim3(k_chunks, m_tiles), 256, 0, st>>>(reinterpret_cast<const __nv_bfloat16*>(w), rows, nullptr, 0, nullptr, 0, K, k_chunks, a_p);

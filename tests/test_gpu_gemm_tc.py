@@ -41,3 +41,29 @@ def test_gemm_tc_rejects_bad_sizes():
     w, a = _case(128, 128, 300, 7)
     with pytest.raises(TB.TabedError):
         TB.debug_gemm_tc(w.to(dev), a.to(dev), 1)          # more than 256 slots per launch
+
+
+def test_a_stand_alone_run_leaves_other_handles_launches_alone():
+    """The limit on a kernel's shared memory is the process's: a small stand-alone product must not lower it below what the
+    LM head of 60 rows takes."""
+    from paper_2601_20357_b200 import binding as TB
+    from paper_2601_20357_b200 import workloads as W
+    dev = torch.device("cuda", 0)
+    cfg = W.DrafterCfg(1, 256, 4, 4, 512, 1000, "bf16")
+    wl = W.Workload(name="limit", config_id=92, drafter=cfg, n_inputs=3, n_requests=20, gamma=1, window_h=4, rounds=1,
+                    policy=W.POLICY_STATIC, prefixes=((("tokens", 1),),) * 3, kv_capacity=16, alpha=(1 / 3,) * 3)
+    g = TB.Tabed(n_inputs=3, n_requests=20, gamma=1, window_h=4, policy=wl.policy, vocab=cfg.vocab, drafter=cfg,
+                 weights=TB.weights_to_device(cfg, W.make_weights(wl), dev), kv_capacity=16)
+    tok, out = torch.zeros(20, dtype=torch.int32, device=dev), torch.empty((60, cfg.vocab), device=dev)
+    saved = g.state_export()
+    seen = []
+    for small in (False, True):
+        if small:
+            w, a = _case(128, 128, 5, 3)
+            TB.debug_gemm_tc(w.to(dev), a.to(dev), 1)
+        g.state_import(saved)
+        g.decode_step(tok, out.fill_(-1.0))
+        torch.cuda.synchronize()
+        seen.append(out.cpu().numpy())
+    assert np.array_equal(seen[0], seen[1])
+    g.destroy()
