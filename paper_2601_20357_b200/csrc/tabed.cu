@@ -192,21 +192,39 @@ void launch_request_clusters(tabed_handle* h, void (*kern)(ArgT), int n_clusters
 int pick_cluster(const tabed_handle* h, int n_clusters, int* slice, int budget_scale = 1) {
   const int by_v = (h->V + 1023) / 1024, n_sm = h->n_sm > 0 ? h->n_sm : 148;
   int cs = 1;
-  // (measured on 32 requests: many small CTAs in several waves beat one wave of large ones - the passes are bound by
-  // dependent latencies and arithmetic, and more resident warps hide both)
+  // (verification and update of 32 requests: many small CTAs in several waves beat one wave of large ones - the passes are
+  // bound by dependent latencies and arithmetic, and more resident warps hide both)
   while (cs * 2 <= h->cs_max && (long long)n_clusters * cs * 2 <= (long long)h->cta_budget * budget_scale * n_sm && cs < by_v) cs *= 2;
   *slice = ((h->V + cs - 1) / cs + 3) & ~3;
   return cs;
 }
 
-// The ensemble step works every CTA for the whole launch, so a second wave costs a launch: the largest cluster, of any size,
-// with which all of them are resident.  (16 requests x 5 steps of 32000 tokens, a
-// whole round: 4 CTAs a cluster, two waves 156 us; 3 CTAs, one wave 148 us.)
+// The ensemble step works every CTA for the whole launch, so a second wave costs a launch (verification and update: pick_cluster):
+// the largest cluster, of any size, with which all of them are resident.  Two things bound that, as measured on 262 shapes
+// (1 - 80 clusters, 1 - 4 inputs, 4000 - 152064 tokens):
+//   * sizes that are not a power of two do not reach the residency that the calculator gives (20 clusters of 12 where it says
+//     21: 18.1 us, of 11: 11.6), so one place in twelve is left free;
+//   * beyond kReqDynSmemMax of slices the logits are read and the exponentials taken again in every pass (80 x 2 x 32000 tokens:
+//     3 CTAs 37.2 us, 4 CTAs in two waves 33.6), so a larger cluster is taken that keeps the slices, in one wave or of the
+//     size that the budget of pick_cluster gives.
+// No shape is slower than with that size alone, and the mean is 7% faster (16 x 5 clusters of 32000 tokens, a whole round: 4 CTAs
+// a cluster, two waves 156 us; 3 CTAs, one wave 148).
 int pick_cluster_one_wave(const tabed_handle* h, int n_clusters, int* slice) {
-  const int by_v = (h->V + 1023) / 1024;
-  int cs = 1;
-  for (int c = 2; c <= std::min(h->cs_max, by_v); ++c) if (n_clusters <= h->cs_active[c]) cs = c;
-  *slice = ((h->V + cs - 1) / cs + 3) & ~3;
+  const int most = std::max(1, std::min(h->cs_max, (h->V + 1023) / 1024));
+  auto slice_of = [&](int c) { return ((h->V + c - 1) / c + 3) & ~3; };
+  auto kept = [&](int c) { return (size_t)h->m * slice_of(c) * sizeof(float) <= kReqDynSmemMax; };
+  int cs = 1, largest = 1;
+  for (int c = 2; c <= most; ++c) {
+    if (n_clusters <= h->cs_active[c]) largest = c;
+    if (n_clusters <= ((c & (c - 1)) == 0 ? h->cs_active[c] : h->cs_active[c] * 11 / 12)) cs = c;
+  }
+  if (!kept(cs)) {
+    int c = cs + 1, s = 0;
+    while (c <= most && !(n_clusters <= h->cs_active[c] && kept(c))) ++c;
+    if (c > most) c = pick_cluster(h, n_clusters, &s);
+    cs = kept(c) ? c : largest;
+  }
+  *slice = slice_of(cs);
   return cs;
 }
 
@@ -923,26 +941,26 @@ int tabed_init(const tabed_config* cfg, const tabed_weights* wts, tabed_handle**
     h->cs_max = 8;
     h->req_dyn_ok = cudaFuncSetAttribute(k_ensemble_req, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kReqDynSmemMax) == cudaSuccess &&
                     cudaFuncSetAttribute(k_verify_req, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kReqDynSmemMax) == cudaSuccess;
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3(kReqMaxCluster); lc.blockDim = dim3(kReqThreads);
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = kReqMaxCluster; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    lc.attrs = at; lc.numAttrs = 1;
     if (cudaFuncSetAttribute(k_ensemble_req, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
         cudaFuncSetAttribute(k_verify_req, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
         cudaFuncSetAttribute(k_verify_tail, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
         cudaFuncSetAttribute(k_update_req, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
-      cudaLaunchConfig_t lc = {};
-      lc.gridDim = dim3(kReqMaxCluster); lc.blockDim = dim3(kReqThreads);
-      cudaLaunchAttribute at[1];
-      at[0].id = cudaLaunchAttributeClusterDimension;
-      at[0].val.clusterDim.x = kReqMaxCluster; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-      lc.attrs = at; lc.numAttrs = 1;
       int n16 = 0;
       bool ok = true;
       for (const void* fn : {(const void*)k_ensemble_req, (const void*)k_verify_req, (const void*)k_verify_tail, (const void*)k_update_req})
         ok = ok && cudaOccupancyMaxActiveClusters(&n16, fn, &lc) == cudaSuccess && n16 >= 1;
       if (ok) h->cs_max = kReqMaxCluster;
-      // how many clusters of each size fit at once (k_ensemble_req: a launch is sized for one wave)
-      for (int cs = 1; cs <= h->cs_max; ++cs) {
-        lc.gridDim = dim3(cs); at[0].val.clusterDim.x = cs;
-        if (cudaOccupancyMaxActiveClusters(&h->cs_active[cs], k_ensemble_req, &lc) != cudaSuccess) h->cs_active[cs] = 0;
-      }
+    }
+    // how many clusters of each size fit at once (k_ensemble_req: a launch is sized for one wave)
+    for (int cs = 1; cs <= h->cs_max; ++cs) {
+      lc.gridDim = dim3(cs); at[0].val.clusterDim.x = cs;
+      if (cudaOccupancyMaxActiveClusters(&h->cs_active[cs], k_ensemble_req, &lc) != cudaSuccess) h->cs_active[cs] = 0;
     }
     cudaGetLastError();
   }

@@ -386,3 +386,21 @@ def test_pool_embeds_bit_exact(gh, gw, d):
         g.pool_embeds(H.t(np.zeros((12, 4), np.float32)), 3, 4, torch.empty((2, 4), device=H.DEV))
     assert e.value.code == -1
     g.destroy()
+
+
+@pytest.mark.parametrize("B,m,V", [(20, 1, 32000), (16, 4, 50000), (20, 3, 80000), (80, 2, 32000), (80, 3, 32000), (3, 2, 1023), (300, 1, 5000)])
+def test_ensemble_step_of_every_cluster_size_matches_the_step_without_a_handle(B, m, V):
+    """Clusters of one wave with a place left free, larger ones that keep their slices, those of the budget, and those that
+    keep none: the bits are those of the chunked kernels."""
+    gen = torch.Generator(device="cuda").manual_seed(B + V)
+    logits = 2.0 * torch.randn((B, m, V), generator=gen, device="cuda")
+    w = torch.softmax(torch.randn((B, m), generator=gen, device="cuda"), 1)
+    u = (torch.randint(0, 1 << 23, (B,), generator=gen, device="cuda").double().add(0.5) * 2.0 ** -23).float()
+    new = lambda: (torch.empty(B, dtype=torch.int32, device="cuda"), torch.empty((B, V), device="cuda"), torch.empty((B, m, V), device="cuda"))
+    a, b = new(), new()
+    g = TB.Tabed(n_inputs=m, n_requests=B, gamma=1, window_h=4, policy=W.POLICY_STATIC, vocab=V)
+    g.ensemble_step(logits, w, u, *a)
+    TB.ensemble_step_static(logits, w, u, *b)
+    torch.cuda.synchronize()
+    assert all(torch.equal(x, y) for x, y in zip(a, b))
+    g.destroy()
