@@ -189,8 +189,6 @@ k_attn_tc_bf16(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
     if (A.act_out) {
       const int k = head * HD + 2 * lane;          // column of the projection's input
       *reinterpret_cast<uint32_t*>(A.act_out + tc_act_offset(s, k, A.act_npad, A.act_chunks) + (k & 7) * 2) = pack_bf16(x0, x1);
-      // an odd number of heads ends in the middle of a block: its other half is this slot's too
-      if (head == H - 1 && (H & 1)) *reinterpret_cast<uint32_t*>(A.act_out + tc_act_offset(s, k + HD, A.act_npad, A.act_chunks) + (k & 7) * 2) = 0u;
     } else {
       *reinterpret_cast<float2*>(A.out + ((size_t)s * H + head) * HD + 2 * lane) = make_float2(x0, x1);
     }

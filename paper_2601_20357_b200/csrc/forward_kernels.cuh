@@ -614,9 +614,6 @@ k_attn_split_bf16(const float* __restrict__ qkv, const SlotDesc* __restrict__ sl
 // Operand blocks of the tensor-core projections for any number of slots: slots are cut into tiles of n_pad (a multiple of
 // 16, at most 256), a tile is k_chunks blocks of 128 columns in the canonical K-major no-swizzle layout (8 rows x 16 bytes
 // core matrices).  Byte offset of the 16-byte piece that holds (slot, columns k .. k + 7).
-// Whoever writes a slot writes ALL its columns, zeros beyond the operand's last one: the buffer is shared by layouts with
-// different n_pad, so a byte that nobody writes in this layout may hold another slot's value of the one before, and where
-// that is not finite its product with the zero weight would be NaN in this slot.
 __host__ __device__ inline size_t tc_act_offset(int slot, int k, int n_pad, int k_chunks) {
   const int t = slot / n_pad, r = slot - t * n_pad;
   return ((size_t)t * k_chunks + k / 128) * ((size_t)n_pad * 256) + ((size_t)((k % 128) >> 3) * (n_pad >> 3) + (r >> 3)) * 128 + (r & 7) * 16;
@@ -644,12 +641,8 @@ __global__ void k_attn_merge(const SlotDesc* __restrict__ slots, int H, int spli
     den = fmaf(f, part_ml[(base + j) * 2 + 1], den);
   }
   const int k = head * HD + dd;
-  if (act_out) {
-    *reinterpret_cast<__nv_bfloat16*>(act_out + tc_act_offset(s, k, act_npad, act_chunks) + (k & 7) * 2) = __float2bfloat16_rn(num / den);
-    if (head == H - 1)                                           // the columns beyond the last head
-      for (int z = k + HD; z < act_chunks * 128; z += HD)
-        *reinterpret_cast<__nv_bfloat16*>(act_out + tc_act_offset(s, z, act_npad, act_chunks) + (z & 7) * 2) = __float2bfloat16_rn(0.0f);
-  } else out[(long long)s * H * HD + k] = num / den;
+  if (act_out) *reinterpret_cast<__nv_bfloat16*>(act_out + tc_act_offset(s, k, act_npad, act_chunks) + (k & 7) * 2) = __float2bfloat16_rn(num / den);
+  else out[(long long)s * H * HD + k] = num / den;
 }
 
 }  // namespace tabed

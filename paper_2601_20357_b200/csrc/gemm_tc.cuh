@@ -41,7 +41,7 @@ struct TcGemmArgs {
   int rows_total;                  // output rows of the projection (multiple of 128 after padding in a_packed)
   int rows_valid;                  // rows actually stored
   int n_pad, n_slots;              // MMA N (multiple of 16) / slots stored
-  int k_chunks;                    // chunks of 128 columns over the whole input dimension
+  int K, k_chunks;                 // the input dimension, and its chunks of 128 columns
   int ks;                          // k-splits; unit (m_tile, split) covers chunks [split*cps, min((split+1)*cps, k_chunks))
   int cps;                         // chunks per split
   int kc;                          // input columns per pipeline stage: 128 (a whole block) or 64 (half a block: a block's
@@ -129,8 +129,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_gemm_tc(const TcGemmArgs G) {
       const uint32_t a_s = smem_u32(tc_smem + (size_t)s * (a_bytes + b_bytes));
       const uint32_t b_s = a_s + (uint32_t)a_bytes;
       const uint32_t a_lbo = (kTcM / 8) * 128, b_lbo = (uint32_t)(G.n_pad / 8) * 128;
+      const int steps = tc_k_steps(G.K, c_lo * kTcKC + c * G.kc, G.kc);
 #pragma unroll 1
-      for (int j = 0; j < G.kc / 16; ++j) {
+      for (int j = 0; j < steps; ++j) {
         const uint64_t da = tc_smem_desc(a_s + (uint32_t)j * 2u * a_lbo, a_lbo, 128u);
         const uint64_t db = tc_smem_desc(b_s + (uint32_t)j * 2u * b_lbo, b_lbo, 128u);
         const uint32_t acc = (c > 0 || j > 0) ? 1u : 0u;

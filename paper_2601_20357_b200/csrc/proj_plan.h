@@ -21,6 +21,14 @@ constexpr int kTcMaxN = 256;       // slots per launch (MMA N is their count rou
 // element (r, k) at ((k/8) * (rows/8) + r/8) * 128 + (r%8) * 16 + (k%8) * 2 bytes.
 TABED_HD inline size_t tc_block_bytes(int rows) { return (size_t)rows * kTcKC * 2; }
 
+// MMAs of 16 columns in a stage of `kc` columns that starts at column k0 of K.  The products stop there: in the activations'
+// blocks nobody writes the columns beyond K (to the next 16), and since the buffer is shared by layouts with different
+// n_pad, another slot's value may lie in them - one that is not finite would turn its zero weight into a NaN of this slot.
+TABED_HD inline int tc_k_steps(int K, int k0, int kc) {
+  const int left = (K - k0 + 15) / 16;
+  return left < kc / 16 ? left : kc / 16;
+}
+
 // Columns of tensor memory that the accumulator of n_pad slots takes (powers of two from 32 on).
 TABED_HD inline int tc_tmem_cols(int n_pad) { return n_pad <= 32 ? 32 : (n_pad <= 64 ? 64 : (n_pad <= 128 ? 128 : 256)); }
 // An allocation of tensor memory waits until the SM has the columns, without a limit, and a CTA of a cluster that waits there

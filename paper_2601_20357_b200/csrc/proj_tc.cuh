@@ -32,7 +32,7 @@ enum ProjEpi { PROJ_QKV = 0, PROJ_RESID = 1, PROJ_SWIGLU = 2 };
 
 struct ProjArgs {
   const unsigned char* a_packed;      // weights [m_tiles][k_chunks] blocks of 128 rows
-  int k_chunks, ks, cps;              // cluster of ks CTAs; CTA r covers chunks [r * cps, min((r + 1) * cps, k_chunks))
+  int K, k_chunks, ks, cps;           // input columns; cluster of ks CTAs; CTA r covers chunks [r * cps, min((r + 1) * cps, k_chunks))
   int n_stages;                       // stages of the weight ring
   unsigned recv_off;                  // > 0: offset of the receive buffer for the other CTAs' slabs (they push); 0: slabs are pulled
   const SlotDesc* slots;
@@ -81,7 +81,7 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_proj_tc(const ProjArgs P) {
   const int split = (int)cluster.block_rank(), m_tile = blockIdx.x / P.ks;
   const int slot0 = blockIdx.y * P.n_pad, n_here = min(P.n_pad, P.n_slots - slot0);
   const int c_lo = split * P.cps, c_hi = min(c_lo + P.cps, P.k_chunks), n_ch = c_hi - c_lo;   // (the host leaves no split empty)
-  const int n_stages = P.n_stages;
+  const int n_stages = P.n_stages, last_steps = tc_k_steps(P.K, (c_hi - 1) * kTcKC, kTcKC);
   const unsigned a_bytes = (unsigned)tc_block_bytes(kTcM), b_bytes = P.x ? proj_norm_block_bytes(P.n_pad) : (unsigned)tc_block_bytes(P.n_pad);
   const uint32_t tmem_cols = (uint32_t)tc_tmem_cols(P.n_pad);
   unsigned char* a_ring = pj_smem;
@@ -195,8 +195,9 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_proj_tc(const ProjArgs P) {
       const uint32_t a_lbo = (kTcM / 8) * 128, b_lbo = (uint32_t)P.n_pad * 16u + (P.x ? 16u : 0u);
       uint64_t da = tc_smem_desc(smem_u32(a_ring + (size_t)s * a_bytes), a_lbo, 128u);
       uint64_t db = tc_smem_desc(smem_u32(b_area + (size_t)(P.x ? c : s) * b_bytes), b_lbo, 128u);
+      const int steps = c == n_ch - 1 ? last_steps : kTcKC / 16;
 #pragma unroll 1
-      for (int j = 0; j < kTcKC / 16; ++j) {
+      for (int j = 0; j < steps; ++j) {
         const uint32_t acc = (c > 0 || j > 0) ? 1u : 0u;
         asm volatile(
             "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
@@ -414,12 +415,11 @@ __global__ void __launch_bounds__(128) k_prep_row(const PrepRowArgs P) {
   if (P.slots && !P.slots[s].active) return;
   const float sc = proj_rms_scale(P.ss + (size_t)s * P.n_ss, P.n_ss, P.d, P.eps);
   const float* xr = P.x + (size_t)s * P.d;
-  for (int k = threadIdx.x * 8; k < P.k_chunks * kTcKC; k += 128 * 8) {
-    uint4 v = make_uint4(0u, 0u, 0u, 0u);                      // (beyond d: tc_act_offset)
-    if (k >= P.d) { *reinterpret_cast<uint4*>(P.dst + tc_act_offset(r, k, P.n_pad, P.k_chunks)) = v; continue; }
+  for (int k = threadIdx.x * 8; k < P.d; k += 128 * 8) {
     const float4 a = *reinterpret_cast<const float4*>(xr + k), b = *reinterpret_cast<const float4*>(xr + k + 4);
     float g[8];
     Elem<__nv_bfloat16>::unpack(__ldg(reinterpret_cast<const uint4*>(P.gain + k)), g);
+    uint4 v;
     v.x = pack_bf16(a.x * sc * g[0], a.y * sc * g[1]); v.y = pack_bf16(a.z * sc * g[2], a.w * sc * g[3]);
     v.z = pack_bf16(b.x * sc * g[4], b.y * sc * g[5]); v.w = pack_bf16(b.z * sc * g[6], b.w * sc * g[7]);
     *reinterpret_cast<uint4*>(P.dst + tc_act_offset(r, k, P.n_pad, P.k_chunks)) = v;

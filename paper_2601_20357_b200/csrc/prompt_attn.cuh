@@ -207,12 +207,6 @@ __global__ void __launch_bounds__(QW * 32 * prompt_attn_groups<HD, QW>(), 1) k_p
     if (r0 < A.n) *reinterpret_cast<uint32_t*>(A.act_out + tc_act_offset(r0, k, A.act_npad, A.act_chunks) + (k & 7) * 2) = pack_bf16(v.x, v.y);
     if (r1 < A.n) *reinterpret_cast<uint32_t*>(A.act_out + tc_act_offset(r1, k, A.act_npad, A.act_chunks) + (k & 7) * 2) = pack_bf16(v.z, v.w);
   }
-  // the columns beyond the last head belong to its CTA (pieces of 8 columns)
-  if (head == A.H - 1)
-    for (int k = A.H * HD + (int)(threadIdx.x / kPaQ) * 8; k < A.act_chunks * 128; k += (int)(blockDim.x / kPaQ) * 8) {
-      const int r = q0 + threadIdx.x % kPaQ;
-      if (r < A.n) *reinterpret_cast<uint4*>(A.act_out + tc_act_offset(r, k, A.act_npad, A.act_chunks)) = make_uint4(0u, 0u, 0u, 0u);
-    }
 }
 
 }  // namespace tabed

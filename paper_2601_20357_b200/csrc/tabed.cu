@@ -667,7 +667,7 @@ int setup_tc(tabed_handle* h) {
   auto A2 = [&](auto** ptr, size_t count, bool zero) { if (rc == TABED_OK) rc = dev_alloc(h, ptr, count, zero); };
   const size_t S2 = (size_t)h->slot_cap * 3 / 2 + kTcMaxN, n_ss = proj_n_ss(h);       // (tiles of at least 32 slots, padded to 16)
   A2(&h->tc_w, h->tc_off[KIND_LM] + h->tck[KIND_LM].bytes, false);
-  // (slots that nobody writes only reach outputs that nobody reads; a slot's columns beyond the operand's K are its writer's)
+  // (slots that nobody writes only reach outputs that nobody reads; the products stop at the operand's last column)
   A2(&h->tc_act, S2 * std::max(h->tck[KIND_QKV].k_chunks, h->tck[KIND_O].k_chunks) * kTcKC * 2, true);
   A2(&h->tc_mid, S2 * h->tck[KIND_DN].k_chunks * kTcKC * 2, true);
   A2(&h->tc_ss_a, n_ss * h->slot_cap, true); A2(&h->tc_ss_m, n_ss * h->slot_cap, true);
@@ -697,7 +697,7 @@ void launch_lm_head_tc(tabed_handle* h, const unsigned char* act, int n, int n_p
   TcGemmArgs G{};
   G.a_packed = h->tc_w + h->tc_off[KIND_LM]; G.b_packed = act; G.partial = logits;
   G.rows_total = t.rows; G.rows_valid = h->V; G.n_pad = n_pad; G.n_slots = n;
-  G.k_chunks = t.k_chunks; G.ks = 1; G.cps = t.k_chunks; G.err = h->err;
+  G.K = t.K; G.k_chunks = t.k_chunks; G.ks = 1; G.cps = t.k_chunks; G.err = h->err;
   G.kc = kTcKC; G.n_stages = tc_stages(n_pad);
   // More tiles than SMs: stages of half a block, so that two CTAs share an SM and one's epilogue overlaps the other's
   // copies (32000 x 768 for 96 slots: 28.8 -> 23.3 us)
@@ -724,7 +724,7 @@ template <int EPI>
 void launch_proj(tabed_handle* h, int kind, int layer, int n_slots, const ProjPlan& p, ProjArgs a) {
   const tabed_handle::TcKind& t = h->tck[kind];
   a.a_packed = h->tc_w + h->tc_off[kind] + (size_t)layer * h->tc_layer_stride;
-  a.k_chunks = t.k_chunks; a.ks = p.ks; a.cps = p.cps; a.n_stages = p.n_stages; a.recv_off = p.recv_off;
+  a.K = t.K; a.k_chunks = t.k_chunks; a.ks = p.ks; a.cps = p.cps; a.n_stages = p.n_stages; a.recv_off = p.recv_off;
   a.slots = h->slots; a.n_slots = n_slots; a.n_pad = p.n_pad; a.err = h->err;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(t.m_tiles * p.ks), (unsigned)p.n_tiles); cfg.blockDim = dim3(kTcThreads);
@@ -1664,7 +1664,7 @@ int tabed_debug_gemm_tc(const void* w, const float* act, int32_t rows, int32_t K
     k_prep_act<<<k_chunks, 256, 0, st>>>(act, K, n, n_pad, K, b_p);
     TcGemmArgs G{};
     G.a_packed = a_p; G.b_packed = b_p; G.partial = part; G.slab = (size_t)n * rows; G.rows_total = rows; G.rows_valid = rows; G.n_pad = n_pad; G.n_slots = n;
-    G.k_chunks = k_chunks; G.ks = ks; G.cps = cps; G.err = err;
+    G.K = K; G.k_chunks = k_chunks; G.ks = ks; G.cps = cps; G.err = err;
     G.kc = kTcKC; G.n_stages = tc_stages(n_pad);
     k_gemm_tc<<<m_tiles * ks, kTcThreads, smem, st>>>(G);
     const size_t elems = (size_t)n * rows;
