@@ -31,6 +31,7 @@ namespace tabed {
 enum ProjEpi { PROJ_QKV = 0, PROJ_RESID = 1, PROJ_SWIGLU = 2 };
 
 struct ProjArgs {
+  int epi;                            // ProjEpi
   const unsigned char* a_packed;      // weights [m_tiles][k_chunks] blocks of 128 rows
   int K, k_chunks, ks, cps;           // input columns; cluster of ks CTAs; CTA r covers chunks [r * cps, min((r + 1) * cps, k_chunks))
   int n_stages;                       // stages of the weight ring
@@ -68,8 +69,9 @@ __device__ __forceinline__ float proj_rms_scale(const float* __restrict__ ss_row
 // (packed: one per stage; RMSNorm: all cps of them) and the receive buffer [ks][owned slots][128] fp32; without room for
 // that (recv_off = 0) a CTA leaves its slab [n_pad][128] over the operands and the others read it from there.
 // The code runs once per launch, so what it costs is trips to L2 and instruction fetch: loads that do not depend on one
-// another are issued together, and loops stay loops.
-template <int EPI>
+// another are issued together, loops stay loops, and the three epilogues are branches of ONE kernel: its code is still in the
+// instruction caches from the launch before, which three instantiations pushed out for one another (a layer of 256 columns and
+// 39 rows 35.2 -> 30.1 us, of 768 columns and 18 rows 49.4 -> 45.8).
 __global__ void __launch_bounds__(kTcThreads, 2) k_proj_tc(const ProjArgs P) {
   namespace cg = cooperative_groups;
   extern __shared__ __align__(128) unsigned char pj_smem[];
@@ -78,7 +80,7 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_proj_tc(const ProjArgs P) {
   __shared__ int s_bad;
   cg::cluster_group cluster = cg::this_cluster();
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int split = (int)cluster.block_rank(), m_tile = blockIdx.x / P.ks;
+  const int epi = P.epi, split = (int)cluster.block_rank(), m_tile = blockIdx.x / P.ks;
   const int slot0 = blockIdx.y * P.n_pad, n_here = min(P.n_pad, P.n_slots - slot0);
   const int c_lo = split * P.cps, c_hi = min(c_lo + P.cps, P.k_chunks), n_ch = c_hi - c_lo;   // (the host leaves no split empty)
   const int n_stages = P.n_stages, last_steps = tc_k_steps(P.K, (c_hi - 1) * kTcKC, kTcKC);
@@ -138,7 +140,7 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_proj_tc(const ProjArgs P) {
       return;
     }
   }
-  if (EPI != PROJ_RESID && P.x) {
+  if (epi != PROJ_RESID && P.x) {
     // RMSNorm prologue.  Warp w takes slots w, w + 8, ...; a unit is one slot's 128 columns of a chunk = one warp-wide
     // 512-byte load (4 columns per lane), eight units and the slots' sums of squares in flight together.
     float scale = 0.0f;                                        // lane i: slot warp + 8 i
@@ -229,8 +231,8 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_proj_tc(const ProjArgs P) {
   __syncwarp();
   // What the epilogue of the warp's first slots reads besides the product is requested before the wait for the product.
   const int o = m_tile * kTcM + lane * 4;
-  const int half = P.hd >> 1, head = EPI == PROJ_QKV ? o / P.hd : 0, hi = EPI == PROJ_QKV ? o - head * P.hd : 0;
-  const bool in_rows = EPI == PROJ_SWIGLU || o < P.rows;
+  const int half = P.hd >> 1, head = epi == PROJ_QKV ? o / P.hd : 0, hi = epi == PROJ_QKV ? o - head * P.hd : 0;
+  const bool in_rows = epi == PROJ_SWIGLU || o < P.rows;
   // The warp's j-th slot of the tile: slot_of(j) = (8 j + warp) ks + split (slots are dealt to the cluster's CTAs, a CTA's to
   // its warps).  Lane j holds the slot's table entry, so that no further trip to L2 is needed for it.
   auto slot_of = [&](int j) { return (j * 8 + warp) * P.ks + split; };
@@ -242,11 +244,11 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_proj_tc(const ProjArgs P) {
 #pragma unroll
     for (int q = 0; q < kBatch; ++q) {
       e0[q] = e1[q] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-      if (EPI == PROJ_SWIGLU) continue;
+      if (epi == PROJ_SWIGLU) continue;
       const int sl = slot_of(j0 + q), pos = __shfl_sync(0xffffffffu, sd.y, j0 + q);
       if (sl >= n_here || !in_rows) continue;
-      if (EPI == PROJ_RESID) e0[q] = *reinterpret_cast<const float4*>(P.x_out + (size_t)(slot0 + sl) * P.rows + o);
-      if (EPI == PROJ_QKV && head < P.H + P.Hkv && pos < P.cap) {      // (a slot past the capacity is inactive)
+      if (epi == PROJ_RESID) e0[q] = *reinterpret_cast<const float4*>(P.x_out + (size_t)(slot0 + sl) * P.rows + o);
+      if (epi == PROJ_QKV && head < P.H + P.Hkv && pos < P.cap) {      // (a slot past the capacity is inactive)
         const size_t at = (size_t)pos * half + (hi < half ? hi : hi - half);
         e0[q] = __ldg(reinterpret_cast<const float4*>(P.rope_cos + at));
         e1[q] = __ldg(reinterpret_cast<const float4*>(P.rope_sin + at));
@@ -307,8 +309,8 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_proj_tc(const ProjArgs P) {
   unsigned char* act_dst = nullptr;
   size_t act_tile = 0;
   int act_r = 0;
-  const float act_inv = EPI == PROJ_SWIGLU ? 1.0f / (float)P.act_npad : 0.0f;
-  if (EPI == PROJ_SWIGLU) {
+  const float act_inv = epi == PROJ_SWIGLU ? 1.0f / (float)P.act_npad : 0.0f;
+  if (epi == PROJ_SWIGLU) {
     const int f = m_tile * (kTcM / 2) + (lane & 15) * 4 + (lane >> 4) * 2, t0 = slot0 / P.act_npad;
     act_tile = (size_t)P.act_chunks * tc_block_bytes(P.act_npad);
     act_r = slot0 - t0 * P.act_npad;
@@ -337,7 +339,7 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_proj_tc(const ProjArgs P) {
         }
       }
     }
-    if (EPI == PROJ_RESID) {
+    if (epi == PROJ_RESID) {
       float ss[kBatch];
 #pragma unroll
       for (int q = 0; q < kBatch; ++q) {
@@ -350,7 +352,7 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_proj_tc(const ProjArgs P) {
 #pragma unroll
       for (int q = 0; q < kBatch; ++q)
         if (lane == 0 && on[q]) P.ss_out[(size_t)(slot0 + slot_of(j0 + q)) * P.n_ss + m_tile] = ss[q];
-    } else if (EPI == PROJ_QKV) {
+    } else if (epi == PROJ_QKV) {
       // rotation pairs are half a head apart; heads do not straddle tiles (hd divides 128)
       const bool rot = head < P.H + P.Hkv;
       const float sgn = hi < half ? -1.0f : 1.0f;

@@ -645,8 +645,7 @@ int setup_tc(tabed_handle* h) {
   h->tc_off[KIND_LM] = h->tc_layer_stride * h->L;
   if (std::max(kTcMaxSmem, kProjMaxSmem) > (size_t)prop.sharedMemPerBlockOptin) return TABED_OK;
   auto smem_attr = [](auto kern, size_t bytes) { return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess; };
-  if (!smem_attr(k_gemm_tc, kTcMaxSmem) || !smem_attr(k_proj_tc<PROJ_QKV>, kProjMaxSmem) || !smem_attr(k_proj_tc<PROJ_RESID>, kProjMaxSmem) ||
-      !smem_attr(k_proj_tc<PROJ_SWIGLU>, kProjMaxSmem) || !smem_attr(k_prompt_attn<32, 4, 64>, prompt_attn_smem<32, 4, 64>()) ||
+  if (!smem_attr(k_gemm_tc, kTcMaxSmem) || !smem_attr(k_proj_tc, kProjMaxSmem) || !smem_attr(k_prompt_attn<32, 4, 64>, prompt_attn_smem<32, 4, 64>()) ||
       !smem_attr(k_prompt_attn<64, 4, 64>, prompt_attn_smem<64, 4, 64>()) || !smem_attr(k_prompt_attn<128, 4, 64>, prompt_attn_smem<128, 4, 64>()) ||
       !smem_attr(k_prompt_attn<32, 2, 32>, prompt_attn_smem<32, 2, 32>()) || !smem_attr(k_prompt_attn<64, 2, 32>, prompt_attn_smem<64, 2, 32>()) ||
       !smem_attr(k_prompt_attn<128, 2, 32>, prompt_attn_smem<128, 2, 32>()))
@@ -661,7 +660,7 @@ int setup_tc(tabed_handle* h) {
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = (unsigned)ks; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
     lc.attrs = at; lc.numAttrs = 1;
-    if (cudaOccupancyMaxActiveClusters(&h->proj_fit[ks], k_proj_tc<PROJ_QKV>, &lc) != cudaSuccess) return TABED_ERR_CUDA;
+    if (cudaOccupancyMaxActiveClusters(&h->proj_fit[ks], k_proj_tc, &lc) != cudaSuccess) return TABED_ERR_CUDA;
   }
   int rc = TABED_OK;
   auto A2 = [&](auto** ptr, size_t count, bool zero) { if (rc == TABED_OK) rc = dev_alloc(h, ptr, count, zero); };
@@ -720,9 +719,9 @@ const tabed_handle::StepPlan& step_plan(tabed_handle* h, int n_slots) {
   return e;
 }
 
-template <int EPI>
 void launch_proj(tabed_handle* h, int kind, int layer, int n_slots, const ProjPlan& p, ProjArgs a) {
   const tabed_handle::TcKind& t = h->tck[kind];
+  a.epi = kind == KIND_QKV ? PROJ_QKV : (kind == KIND_GU ? PROJ_SWIGLU : PROJ_RESID);
   a.a_packed = h->tc_w + h->tc_off[kind] + (size_t)layer * h->tc_layer_stride;
   a.K = t.K; a.k_chunks = t.k_chunks; a.ks = p.ks; a.cps = p.cps; a.n_stages = p.n_stages; a.recv_off = p.recv_off;
   a.slots = h->slots; a.n_slots = n_slots; a.n_pad = p.n_pad; a.err = h->err;
@@ -735,7 +734,7 @@ void launch_proj(tabed_handle* h, int kind, int layer, int n_slots, const ProjPl
   at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at; cfg.numAttrs = 2;
-  cudaLaunchKernelEx(&cfg, k_proj_tc<EPI>, a);
+  cudaLaunchKernelEx(&cfg, k_proj_tc, a);
   h->launches++;
 }
 
@@ -782,7 +781,7 @@ void run_step_tc(tabed_handle* h, StepArgs sa, int n_slots, int max_pos, float* 
       a.rows = h->qkv_w; a.qkv = h->qkv; a.rope_cos = h->rope_cos; a.rope_sin = h->rope_sin;
       a.kc = reinterpret_cast<bf*>(h->kc); a.vc = reinterpret_cast<bf*>(h->vc);
       a.H = h->H; a.Hkv = h->Hkv; a.hd = h->hd; a.layer = l; a.L = h->L; a.cap = h->cap;
-      launch_proj<PROJ_QKV>(h, KIND_QKV, l, n_slots, pq, a);
+      launch_proj(h, KIND_QKV, l, n_slots, pq, a);
     }
     if (!logits_out && l == h->L - 1) break;
     {
@@ -796,20 +795,20 @@ void run_step_tc(tabed_handle* h, StepArgs sa, int n_slots, int max_pos, float* 
       ProfScope ps(h, TABED_PROF_OPROJ);
       ProjArgs a{};
       a.b_packed = h->tc_act; a.rows = d; a.x_out = h->x; a.ss_out = h->tc_ss_m; a.n_ss = n_ss;
-      launch_proj<PROJ_RESID>(h, KIND_O, l, n_slots, po, a);
+      launch_proj(h, KIND_O, l, n_slots, po, a);
     }
     {
       ProfScope ps(h, TABED_PROF_GATEUP);
       ProjArgs a{};
       normed(a, pg, h->tc_ss_m, h->norm2[l]);
       a.act_out = h->tc_mid; a.act_npad = pd.n_pad; a.act_chunks = h->tck[KIND_DN].k_chunks;
-      launch_proj<PROJ_SWIGLU>(h, KIND_GU, l, n_slots, pg, a);
+      launch_proj(h, KIND_GU, l, n_slots, pg, a);
     }
     {
       ProfScope ps(h, TABED_PROF_DOWN);
       ProjArgs a{};
       a.b_packed = h->tc_mid; a.rows = d; a.x_out = h->x; a.ss_out = h->tc_ss_a; a.n_ss = n_ss;
-      launch_proj<PROJ_RESID>(h, KIND_DN, l, n_slots, pd, a);
+      launch_proj(h, KIND_DN, l, n_slots, pd, a);
     }
   }
   if (logits_out) {
