@@ -28,7 +28,7 @@
 
 namespace tabed {
 
-enum ProjEpi { PROJ_QKV = 0, PROJ_RESID = 1, PROJ_SWIGLU = 2 };
+enum ProjEpi { PROJ_QKV = 0, PROJ_RESID = 1, PROJ_SWIGLU = 2, PROJ_ANY = 3 };
 
 struct ProjArgs {
   int epi;                            // ProjEpi
@@ -69,9 +69,11 @@ __device__ __forceinline__ float proj_rms_scale(const float* __restrict__ ss_row
 // (packed: one per stage; RMSNorm: all cps of them) and the receive buffer [ks][owned slots][128] fp32; without room for
 // that (recv_off = 0) a CTA leaves its slab [n_pad][128] over the operands and the others read it from there.
 // The code runs once per launch, so what it costs is trips to L2 and instruction fetch: loads that do not depend on one
-// another are issued together, loops stay loops, and the three epilogues are branches of ONE kernel: its code is still in the
-// instruction caches from the launch before, which three instantiations pushed out for one another (a layer of 256 columns and
-// 39 rows 35.2 -> 30.1 us, of 768 columns and 18 rows 49.4 -> 45.8).
+// another are issued together, loops stay loops, and the three epilogues are branches of ONE kernel (PROJ_ANY): its code is
+// still in the instruction caches from the launch before, which three instantiations pushed out for one another (a layer of
+// 256 columns and 39 rows 35.2 -> 30.1 us, of 768 columns and 18 rows 49.4 -> 45.8).  Long prompts run the code often enough
+// to gain from instantiations without the branches (step_plan).
+template <int EPI>
 __global__ void __launch_bounds__(kTcThreads, 2) k_proj_tc(const ProjArgs P) {
   namespace cg = cooperative_groups;
   extern __shared__ __align__(128) unsigned char pj_smem[];
@@ -80,7 +82,7 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_proj_tc(const ProjArgs P) {
   __shared__ int s_bad;
   cg::cluster_group cluster = cg::this_cluster();
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int epi = P.epi, split = (int)cluster.block_rank(), m_tile = blockIdx.x / P.ks;
+  const int epi = EPI == PROJ_ANY ? P.epi : EPI, split = (int)cluster.block_rank(), m_tile = blockIdx.x / P.ks;
   const int slot0 = blockIdx.y * P.n_pad, n_here = min(P.n_pad, P.n_slots - slot0);
   const int c_lo = split * P.cps, c_hi = min(c_lo + P.cps, P.k_chunks), n_ch = c_hi - c_lo;   // (the host leaves no split empty)
   const int n_stages = P.n_stages, last_steps = tc_k_steps(P.K, (c_hi - 1) * kTcKC, kTcKC);

@@ -116,7 +116,7 @@ struct tabed_handle {
   unsigned char *tc_act = nullptr, *tc_mid = nullptr;   // operand blocks: normalised rows or attention outputs; gated products
   float *tc_ss_a = nullptr, *tc_ss_m = nullptr;         // partial sums of squares of the residual [slot][n_ss], entering a
                                                         // layer and between its attention and its MLP
-  struct StepPlan { int n_slots; ProjPlan p[4]; };
+  struct StepPlan { int n_slots; ProjPlan p[4]; bool each_its_own; };
   StepPlan step_plans[16]{};        // (n_slots 0: none yet)
   int next_plan = 0;
   int proj_fit[9]{};                // resident clusters of 1 .. 8 CTAs of a projection, one CTA per SM
@@ -645,7 +645,8 @@ int setup_tc(tabed_handle* h) {
   h->tc_off[KIND_LM] = h->tc_layer_stride * h->L;
   if (std::max(kTcMaxSmem, kProjMaxSmem) > (size_t)prop.sharedMemPerBlockOptin) return TABED_OK;
   auto smem_attr = [](auto kern, size_t bytes) { return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess; };
-  if (!smem_attr(k_gemm_tc, kTcMaxSmem) || !smem_attr(k_proj_tc, kProjMaxSmem) || !smem_attr(k_prompt_attn<32, 4, 64>, prompt_attn_smem<32, 4, 64>()) ||
+  if (!smem_attr(k_gemm_tc, kTcMaxSmem) || !smem_attr(k_proj_tc<PROJ_ANY>, kProjMaxSmem) || !smem_attr(k_proj_tc<PROJ_QKV>, kProjMaxSmem) ||
+      !smem_attr(k_proj_tc<PROJ_RESID>, kProjMaxSmem) || !smem_attr(k_proj_tc<PROJ_SWIGLU>, kProjMaxSmem) || !smem_attr(k_prompt_attn<32, 4, 64>, prompt_attn_smem<32, 4, 64>()) ||
       !smem_attr(k_prompt_attn<64, 4, 64>, prompt_attn_smem<64, 4, 64>()) || !smem_attr(k_prompt_attn<128, 4, 64>, prompt_attn_smem<128, 4, 64>()) ||
       !smem_attr(k_prompt_attn<32, 2, 32>, prompt_attn_smem<32, 2, 32>()) || !smem_attr(k_prompt_attn<64, 2, 32>, prompt_attn_smem<64, 2, 32>()) ||
       !smem_attr(k_prompt_attn<128, 2, 32>, prompt_attn_smem<128, 2, 32>()))
@@ -660,7 +661,7 @@ int setup_tc(tabed_handle* h) {
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = (unsigned)ks; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
     lc.attrs = at; lc.numAttrs = 1;
-    if (cudaOccupancyMaxActiveClusters(&h->proj_fit[ks], k_proj_tc, &lc) != cudaSuccess) return TABED_ERR_CUDA;
+    if (cudaOccupancyMaxActiveClusters(&h->proj_fit[ks], k_proj_tc<PROJ_ANY>, &lc) != cudaSuccess) return TABED_ERR_CUDA;
   }
   int rc = TABED_OK;
   auto A2 = [&](auto** ptr, size_t count, bool zero) { if (rc == TABED_OK) rc = dev_alloc(h, ptr, count, zero); };
@@ -716,10 +717,15 @@ const tabed_handle::StepPlan& step_plan(tabed_handle* h, int n_slots) {
   e.p[KIND_O] = plan_proj(h->tck[KIND_O].m_tiles, h->tck[KIND_O].k_chunks, n_slots, false, h->proj_fit);
   e.p[KIND_GU] = plan_proj(h->tck[KIND_GU].m_tiles, h->tck[KIND_GU].k_chunks, n_slots, true, h->proj_fit);
   e.p[KIND_DN] = plan_proj(h->tck[KIND_DN].m_tiles, h->tck[KIND_DN].k_chunks, n_slots, false, h->proj_fit);
+  // which kernels: the one with all epilogues, or one each where several slot tiles and much gate/up work run the code often
+  // (blocks of 128 x 128 weights times slots).  Prompts, one kernel -> one each: 896 columns, 1155 positions 7088 -> 6907 us; 704,
+  // 683 positions 1065 -> 1052; 512, 1006 positions 1202 -> 1212; 256, 865 positions 1628 -> 1691
+  e.each_its_own = n_slots > kTcMaxN && (long long)h->tck[KIND_GU].m_tiles * h->tck[KIND_GU].k_chunks * n_slots > 65536;
   return e;
 }
 
-void launch_proj(tabed_handle* h, int kind, int layer, int n_slots, const ProjPlan& p, ProjArgs a) {
+void launch_proj(tabed_handle* h, int kind, int layer, int n_slots, const tabed_handle::StepPlan& plan, ProjArgs a) {
+  const ProjPlan& p = plan.p[kind];
   const tabed_handle::TcKind& t = h->tck[kind];
   a.epi = kind == KIND_QKV ? PROJ_QKV : (kind == KIND_GU ? PROJ_SWIGLU : PROJ_RESID);
   a.a_packed = h->tc_w + h->tc_off[kind] + (size_t)layer * h->tc_layer_stride;
@@ -734,7 +740,9 @@ void launch_proj(tabed_handle* h, int kind, int layer, int n_slots, const ProjPl
   at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at; cfg.numAttrs = 2;
-  cudaLaunchKernelEx(&cfg, k_proj_tc, a);
+  auto kern = k_proj_tc<PROJ_ANY>;
+  if (plan.each_its_own) kern = a.epi == PROJ_QKV ? k_proj_tc<PROJ_QKV> : (a.epi == PROJ_RESID ? k_proj_tc<PROJ_RESID> : k_proj_tc<PROJ_SWIGLU>);
+  cudaLaunchKernelEx(&cfg, kern, a);
   h->launches++;
 }
 
@@ -781,7 +789,7 @@ void run_step_tc(tabed_handle* h, StepArgs sa, int n_slots, int max_pos, float* 
       a.rows = h->qkv_w; a.qkv = h->qkv; a.rope_cos = h->rope_cos; a.rope_sin = h->rope_sin;
       a.kc = reinterpret_cast<bf*>(h->kc); a.vc = reinterpret_cast<bf*>(h->vc);
       a.H = h->H; a.Hkv = h->Hkv; a.hd = h->hd; a.layer = l; a.L = h->L; a.cap = h->cap;
-      launch_proj(h, KIND_QKV, l, n_slots, pq, a);
+      launch_proj(h, KIND_QKV, l, n_slots, plan, a);
     }
     if (!logits_out && l == h->L - 1) break;
     {
@@ -795,20 +803,20 @@ void run_step_tc(tabed_handle* h, StepArgs sa, int n_slots, int max_pos, float* 
       ProfScope ps(h, TABED_PROF_OPROJ);
       ProjArgs a{};
       a.b_packed = h->tc_act; a.rows = d; a.x_out = h->x; a.ss_out = h->tc_ss_m; a.n_ss = n_ss;
-      launch_proj(h, KIND_O, l, n_slots, po, a);
+      launch_proj(h, KIND_O, l, n_slots, plan, a);
     }
     {
       ProfScope ps(h, TABED_PROF_GATEUP);
       ProjArgs a{};
       normed(a, pg, h->tc_ss_m, h->norm2[l]);
       a.act_out = h->tc_mid; a.act_npad = pd.n_pad; a.act_chunks = h->tck[KIND_DN].k_chunks;
-      launch_proj(h, KIND_GU, l, n_slots, pg, a);
+      launch_proj(h, KIND_GU, l, n_slots, plan, a);
     }
     {
       ProfScope ps(h, TABED_PROF_DOWN);
       ProjArgs a{};
       a.b_packed = h->tc_mid; a.rows = d; a.x_out = h->x; a.ss_out = h->tc_ss_a; a.n_ss = n_ss;
-      launch_proj(h, KIND_DN, l, n_slots, pd, a);
+      launch_proj(h, KIND_DN, l, n_slots, plan, a);
     }
   }
   if (logits_out) {
