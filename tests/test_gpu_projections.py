@@ -56,6 +56,18 @@ def test_prompt_chunks_agree_with_one_position_at_a_time(heads, kv_heads, hd, ff
     assert np.max(np.abs(a - b)) <= 2 * H.logit_tols(wl)[0]
 
 
+@pytest.mark.parametrize("heads,hd,ffn,n", [(8, 128, 4096, 800), (8, 64, 2560, 700)])
+def test_long_prompts_of_wide_drafters_agree_with_one_position_at_a_time(heads, hd, ffn, n):
+    """The forms that only much work takes: a kernel of its own per epilogue; 64 positions a CTA of the prompt attention at a
+    head size of 128; and, at 1024 / 4096 columns and 800 positions, a down projection whose CTAs read one another's partial
+    sums where they lie (tests/test_proj_plan.py checks that the plan is such a one)."""
+    wl = _workload(1, 1, heads, heads, hd, ffn, n + 8)
+    weights = TB.weights_to_device(wl.drafter, W.make_weights(wl), torch.device("cuda", 0))
+    a = _logits_after(wl, weights, TB.PATH_TENSOR_CORE, ((n, 0),), 7)
+    b = _logits_after(wl, weights, TB.PATH_PER_OP, ((n, 0),), 7)
+    assert np.max(np.abs(a - b)) <= 2 * H.logit_tols(wl)[0]
+
+
 @pytest.mark.parametrize("B,m", [(1, 1), (5, 3), (11, 3), (43, 3), (129, 2)])
 def test_rows_at_tile_edges_agree_with_per_operation_step(B, m):
     """1, 15, 33, 129 and 258 rows: one tile and several, whole and ragged (the plan of a projection depends on the count)."""

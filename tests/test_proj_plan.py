@@ -62,3 +62,10 @@ def program(tmp_path_factory):
 def test_plans_keep_to_the_memory_that_a_cta_and_its_neighbours_have(program):
     res = subprocess.run([program], capture_output=True, text=True)
     assert res.returncode == 0, res.stdout
+
+
+def test_a_long_down_projection_pulls_its_partial_sums(program):
+    """1024 columns from 4096 at 800 positions: no room for a receive buffer beside the operands (the GPU test of that form
+    relies on it)."""
+    n_pad, ks, stages, norm, recv_off, smem = map(int, subprocess.run([program, "1024", "4096", "800", "0"], capture_output=True, text=True, check=True).stdout.split())
+    assert ks > 1 and recv_off == 0
