@@ -26,6 +26,10 @@
  *     distribution without mass) set bits in an error word on the device.  tabed_round_host, which
  *     synchronises anyway, returns the matching code (TABED_ERR_TIMEOUT / _KV_OVERFLOW / _NUMERIC) and
  *     clears the word; after the asynchronous calls use tabed_last_device_error.
+ *   - Embeddings, weights and loaded caches are expected to be finite.  The decode kernels read a row's last tile of
+ *     cache positions whole and give the positions beyond its length a weight of zero, so a row that once held
+ *     non-finite positions may give NaN again after tabed_state_import took it back to a shorter length, until
+ *     tabed_load_prefix_kv or a prompt over those positions replaces them.
  *   - Layouts are row-major with the last index fastest.  B = n_requests, m = n_inputs,
  *     R = B*m rows (row = request*m + input), V = vocab, G = gamma.
  *   - Uniforms are caller-supplied floats on the lattice u = (k + 1/2) * 2^-23, 0 <= k < 2^23.
@@ -362,8 +366,10 @@ int tabed_state_import(tabed_handle* h, const void* host, size_t bytes);
  * records a CUDA event pair on config.stream around every launch (group) of that class;
  * tabed_profile_end synchronises the stream and returns the summed elapsed milliseconds and the
  * number of timed intervals.  TABED_PROF_ATTENTION, _ENSEMBLE, _VERIFY and _UPDATE time their group
- * of kernels as one interval; the others time a single kernel per interval.  Classes 0-6 only occur
- * on the per-operation path, TABED_PROF_DRAFT_ROUND only on the persistent path. */
+ * of kernels as one interval (TABED_PROF_ENSEMBLE: one per drafting step, or one for all steps of a round on the
+ * caller's own logits); the others time a single kernel per interval, with the one that packs its input where the
+ * tensor-core path has such a one.  Classes 0-6 occur on the per-operation and tensor-core paths (6 on rounds with
+ * the caller's logits too), TABED_PROF_DRAFT_ROUND only on the persistent path. */
 #define TABED_PROF_QKV        0
 #define TABED_PROF_ATTENTION  1
 #define TABED_PROF_OPROJ      2

@@ -66,7 +66,7 @@ __device__ __forceinline__ bool tc_wait(uint64_t* bar, unsigned parity, int* err
   return true;
 }
 
-// grid (m_tiles * ks), block 128, dynamic shared memory kTcStages * (A block + B block) + 1 KB
+// grid (m_tiles * ks), block kTcThreads, dynamic shared memory n_stages * (A + B of a stage) + 1 KB
 __global__ void __launch_bounds__(kTcThreads, 1) k_gemm_tc(const TcGemmArgs G) {
   extern __shared__ __align__(1024) unsigned char tc_smem[];
   __shared__ uint64_t s_full[kTcMaxStages], s_empty[kTcMaxStages], s_done;

@@ -59,10 +59,14 @@ struct ProjPlan {
 };
 
 // The plan for n_slots slots; fit_of[ks]: clusters of ks CTAs that the device keeps resident at once, one CTA per SM.  What a
-// choice costs, in us, as measured on the kernel's own time line (18 - 1024 slots, 768 - 4864 columns): a CTA draws 75 KB/us alone and all of them together
-// 6.5 MB/us from L2; 8 slots of the epilogue cost each warp 0.2 us; the exchange between the CTAs of a cluster 1 us, and
-// 0.02 us per slot more where the slabs are pulled for lack of a receive buffer; a normalising prologue 1.2 us and 0.02 us per
-// slot and 128 columns, against 3 us for a launch that packs the operand; a wave that is not full costs a wave.
+// choice costs, in us, as measured on the kernel's own time line (18 - 1024 slots, 768 - 4864 columns): 2 us whatever it does;
+// its operands, which a CTA draws from L2 at 75 KB/us alone (60 with a ring of two stages, which does not cover the trip) and
+// all of them together at 6.5 MB/us; 0.25 for every 8 slots of the epilogue; the exchange between the CTAs of a cluster 1 us,
+// and 0.02 per slot more where the slabs are pulled for lack of a receive buffer; a normalising prologue 1.2 us and 0.02 per
+// slot and 128 columns, against 3 us for a launch that packs the operand; a wave that is not full costs a wave; 0.5 us less
+// where half of the shared memory is left for the next kernel's start.  All plans of 12 drafters of 256 - 1024 columns were timed
+// at 3 - 96 rows: nine launches in ten are within 1 us of their best; the worst are down projections of 768 - 1024 columns with
+// two stages in half of the memory (1.5 - 2.7 us slower than three in all of it) and gate/up at 832 columns (2.3 us).
 inline ProjPlan plan_proj(int m_tiles, int k_chunks, int n_slots, bool can_norm, const int* fit_of) {
   ProjPlan best{};
   best.us = 1e30f;

@@ -16,7 +16,8 @@
 //   * RMSNorm is the prologue: the producer leaves one partial sum of squares per (128-row tile, slot), the consumer adds
 //     the few of them, scales, rounds and writes its own columns of the operand straight into shared memory;
 //   * the weights of the first stages are requested before the wait on the kernel before (they depend on nothing).
-// 9 launches a layer became 5 (one of them the attention); measured figures are beside plan_proj and run_step_tc.
+// 9 launches a layer became 5 (one of them the attention): a layer of 768 columns and 18 rows 49.6 -> 40.9 us, 96 rows 78.6 ->
+// 69.2, of 256 columns and 39 rows 32.2 -> 30.5.  What a launch's parts cost stands at plan_proj.
 // Every wait is bounded; on a timeout the CTA sets an error bit, lets its copies land, frees TMEM and leaves.
 #pragma once
 #include <cooperative_groups.h>
@@ -71,7 +72,7 @@ __device__ __forceinline__ float proj_rms_scale(const float* __restrict__ ss_row
 // The code runs once per launch, so what it costs is trips to L2 and instruction fetch: loads that do not depend on one
 // another are issued together, loops stay loops, and the three epilogues are branches of ONE kernel (PROJ_ANY): its code is
 // still in the instruction caches from the launch before, which three instantiations pushed out for one another (a layer of
-// 256 columns and 39 rows 35.2 -> 30.1 us, of 768 columns and 18 rows 49.4 -> 45.8).  Long prompts run the code often enough
+// 256 columns and 39 rows 35.2 -> 30.5 us, of 768 columns and 18 rows 45.8 -> 40.9).  Long prompts run the code often enough
 // to gain from instantiations without the branches (step_plan).
 template <int EPI>
 __global__ void __launch_bounds__(kTcThreads, 2) k_proj_tc(const ProjArgs P) {

@@ -8,7 +8,7 @@
 // weights are split into a bf16 head and a bf16 remainder (two products), so products are exact to ~2^-17 and sums are fp32,
 // as in the decode kernels.  A prompt of 576 positions and 12 heads is 2 GFLOP against 0.9 MB of cache per head: neither
 // roofline is near, what counts is that the K, V tiles are shared by the CTA's positions (the decode kernel reads the cache
-// once per position: 66 us for 256 positions of a 768-wide layer, this one 14 for 576).  The longest CTAs (last positions)
+// once per position).  A launch for 128 positions of a 768-wide layer takes 12.8 us by itself.  The longest CTAs (last positions)
 // start first.  Short prompts would leave most SMs idle with 64 positions a CTA (128 positions x 12 heads: 24 CTAs, whose
 // products then wait for one another on the tensor pipe): where these CTAs fill at most half of the SMs, 32 positions and
 // tiles of 32 in eight groups are taken.

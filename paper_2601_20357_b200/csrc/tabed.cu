@@ -106,7 +106,7 @@ struct tabed_handle {
   bool atc_ok = false; CUtensorMap tm_k, tm_v;
   unsigned char* packed = nullptr;
   unsigned long long* trace = nullptr; int trace_stride = 0; bool trace_on = false; int trace_cta = 0;
-  // tensor-core projections for many rows (bf16 drafter, more than 8 slots per step)
+  // tensor-core projections (bf16 drafter; any number of slots)
   bool tc_ok = false;                        // tcgen05 projections are set up: prompts, single steps, and rounds without the persistent kernel
   int slot_cap = 0;                          // slots the step buffers hold: 2R, or a prefill chunk if that is more
   struct TcKind { int rows, K, m_tiles, k_chunks; size_t bytes; };
@@ -718,8 +718,9 @@ const tabed_handle::StepPlan& step_plan(tabed_handle* h, int n_slots) {
   e.p[KIND_GU] = plan_proj(h->tck[KIND_GU].m_tiles, h->tck[KIND_GU].k_chunks, n_slots, true, h->proj_fit);
   e.p[KIND_DN] = plan_proj(h->tck[KIND_DN].m_tiles, h->tck[KIND_DN].k_chunks, n_slots, false, h->proj_fit);
   // which kernels: the one with all epilogues, or one each where several slot tiles and much gate/up work run the code often
-  // (blocks of 128 x 128 weights times slots).  Prompts, one kernel -> one each: 896 columns, 1155 positions 7088 -> 6907 us; 704,
-  // 683 positions 1065 -> 1052; 512, 1006 positions 1202 -> 1212; 256, 865 positions 1628 -> 1691
+  // (blocks of 128 x 128 weights times slots).  Whole prompts of 3 - 4 inputs, one kernel -> one each: 896 columns, a 32 x 32
+  // image and text 7088 -> 6907 us; 704 columns, 16 x 16 and 427 tokens 1065 -> 1052; 512, 26 x 26 and 330 tokens 1202 -> 1212;
+  // 256, 24 x 24 and 289 tokens 1628 -> 1691
   e.each_its_own = n_slots > kTcMaxN && (long long)h->tck[KIND_GU].m_tiles * h->tck[KIND_GU].k_chunks * n_slots > 65536;
   return e;
 }
@@ -1610,8 +1611,8 @@ int tabed_state_import(tabed_handle* h, const void* host, size_t bytes) {
     }
   }
   DeviceGuard guard(h->cfg.device);
-  // one copy of the whole snapshot and one kernel that deals it to its arrays (a copy per array: a round of the
-  // caller's own logits with its import 148 us, now 141)
+  // one copy of the whole snapshot and one kernel that deals it to its arrays (a copy per array: the import and a round of the
+  // caller's own logits 148 us, now 141)
   SnapParts S{};
   for (const auto& s : parts) {
     S.dst[S.n] = reinterpret_cast<uint32_t*>(s.ptr); S.begin[S.n] = (unsigned)((in - reinterpret_cast<const unsigned char*>(host)) / 4);
