@@ -125,7 +125,7 @@ def test_attention_many_rows_several_chunks_each():
 def test_chunked_prefill_matches_position_by_position_prefill(heads, kv_heads, d):
     """The same prompts (700, 130 and 37 embeddings + 9 tokens: one chunk each) fed as a chunk of positions
     (tcgen05 projections, every position attending up to itself) and one position at a time (per-operation
-    kernels): both handles then follow the checker in lock step, and their first drafting step agrees within
+    kernels): both handles then follow the oracle in lock step, and their first drafting step agrees within
     the bf16 bound.  Head sizes 64 and 32.  (Prompts of several chunks: the next test.)"""
     wl = wl_attn(heads=heads, kv_heads=kv_heads, d=d, cap=1024, cid=120 + heads,
                  prefixes=((("tokens", 700),), (("tokens", 130),), (("embeds", 37), ("tokens", 9))))
@@ -150,7 +150,7 @@ def test_chunked_prefill_matches_position_by_position_prefill(heads, kv_heads, d
         pair.gpu.destroy()
 
 
-def test_prompts_of_several_chunks_follow_the_checker():
+def test_prompts_of_several_chunks_follow_the_oracle():
     """1212 tokens and 1100 embeddings are a full chunk of 1024 positions and a second one each, at an offset into the tokens
     (embeddings) and into the cache, with a slot count of its own; a short prompt between them."""
     wl = wl_attn(heads=4, kv_heads=2, d=256, cap=1300, cid=133, prefixes=((("tokens", 1212),), (("embeds", 37), ("tokens", 9)), (("embeds", 1100),)))
