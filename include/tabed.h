@@ -295,9 +295,9 @@ int tabed_current_path(const tabed_handle* h);
 /* Switch the phase timeline of the persistent kernel off (on = 0) or on (on = 1 + the index of the CTA
  * that records; CTA 0 if the grid is smaller): when on, that CTA stores one record of
  * 8 words per phase into TABED_VIEW_TRACE (first index = drafting step): [0] the GPU's
- * nanosecond timer at the end of the phase; [1..5] SM clock cycles that that CTA spent in the phase
- * waiting for and staging activations, waiting for weight tiles, in the tensor-core products,
- * issuing weight copies and in epilogues, and in the rest (for the phases without weights: all of the
+ * nanosecond timer at the end of the phase (O, down: when their results have arrived); [1..5] SM clock
+ * cycles that that CTA's first warp spent in the phase waiting for activations, in weight tiles and products,
+ * at the barrier behind them, in the epilogue, and in the rest (for the phases of other warps: all of the
  * phase); [6..7] unused.  Phase order within a step: per layer QKV, attention, O, gate/up, down; then
  * LM head, [1 more when tabed_debug_override_logits is set], exp-sum, mix.
  * Errors: UNSUPPORTED (no persistent path). */

@@ -96,8 +96,8 @@ struct tabed_handle {
   unsigned launches_persist = 0;
   LayerW* layer_tab = nullptr;
   // its exchange buffers of flagged words {value, epoch} and the epoch the next launch starts from
-  uint2 *ll_xa = nullptr, *ll_x1 = nullptr, *ll_qkv = nullptr, *ll_mid = nullptr, *ll_po = nullptr, *ll_pml = nullptr;
-  uint2 *ll_rowmax = nullptr, *ll_rowmax2 = nullptr, *ll_rowsum = nullptr, *ll_cmass = nullptr;
+  uint2 *ll_xa = nullptr, *ll_x1 = nullptr, *ll_qkv = nullptr, *ll_att = nullptr, *ll_mid = nullptr, *ll_part = nullptr;
+  uint2 *ll_rowmax = nullptr, *ll_rowsum = nullptr, *ll_slice = nullptr, *ll_mass = nullptr;
   std::vector<std::pair<void*, size_t>> ll_all;       // every exchange buffer (cleared when the epoch counter wraps)
   unsigned ll_epoch = 0;
   uint2* ll_probe = nullptr;        // a word nobody ever writes (tabed_debug_barrier_timeout)
@@ -442,15 +442,23 @@ void run_ensemble(tabed_handle* h, const float* logits, const float* w, const fl
 }
 
 // ---- persistent drafting-round kernel: geometry and set-up -----------------------------------------
-// Cut a [16*n_tiles][K] weight matrix into tiles of 16 rows; a tile whose rows are longer than kcap
-// becomes nsub sub-units (1, 2 or a multiple of 4, so that they line up with the 4 warp groups).
-PhaseGeom pick_geom(int n_tiles, int K, int kcap) {
+// Cut a weight matrix [rows * n_tiles][K] into tiles; a tile whose rows are longer than kcap becomes nsub sub-units.
+PhaseGeom pick_geom(int rows, int n_tiles, int K, int kcap) {
   const int nkb = K / 16;
-  for (int nsub = 1; nsub <= 64; nsub = (nsub < 4) ? nsub * 2 : nsub + 4) {
-    if (nkb % nsub || K / nsub > kcap) continue;
-    return PhaseGeom{n_tiles, nsub, K / nsub, n_tiles * nsub};
-  }
-  return PhaseGeom{n_tiles, 0, 0, 0};
+  for (int nsub = 1; nsub <= 63; ++nsub)
+    if (nkb % nsub == 0 && K / nsub <= kcap) return PhaseGeom{rows, n_tiles, nsub, K / nsub, n_tiles * nsub};
+  return PhaseGeom{rows, n_tiles, 0, 0, 0};
+}
+
+template <int HD>
+const void* draft_round_kernel(int d, bool trace) {
+  if (d <= 6 * 16 * kGW) return trace ? (const void*)k_draft_round<HD, 6, true> : (const void*)k_draft_round<HD, 6, false>;
+  if (d <= 8 * 16 * kGW) return trace ? (const void*)k_draft_round<HD, 8, true> : (const void*)k_draft_round<HD, 8, false>;
+  if (d <= 12 * 16 * kGW) return trace ? (const void*)k_draft_round<HD, 12, true> : (const void*)k_draft_round<HD, 12, false>;
+  return trace ? (const void*)k_draft_round<HD, 24, true> : (const void*)k_draft_round<HD, 24, false>;
+}
+const void* draft_round_kernel(const tabed_handle* h, bool trace) {
+  return h->hd == 32 ? draft_round_kernel<32>(h->d, trace) : (h->hd == 64 ? draft_round_kernel<64>(h->d, trace) : draft_round_kernel<128>(h->d, trace));
 }
 
 // Decides whether the handle's drafter can run on the persistent kernel and allocates its buffers.
@@ -469,48 +477,52 @@ int setup_persistent(tabed_handle* h) {
   cudaDeviceProp prop;
   if (cudaGetDeviceProperties(&prop, c.device) != cudaSuccess) return TABED_ERR_CUDA;
   if (!prop.cooperativeLaunch) return TABED_OK;
+  const void *kern = draft_round_kernel(h, false), *kern_trace = draft_round_kernel(h, true);
   cudaFuncAttributes fa;
-  if (cudaFuncGetAttributes(&fa, k_draft_round<true>) != cudaSuccess) return TABED_ERR_CUDA;
+  if (cudaFuncGetAttributes(&fa, kern_trace) != cudaSuccess) return TABED_ERR_CUDA;
   const int n_cta = prop.multiProcessorCount;
   if (n_cta > kPT) return TABED_OK;
+  if ((kPSlots * h->Hkv * ((h->cap + kPPos - 1) / kPPos) + n_cta - 1) / n_cta + 1 > kPMaxChunks) return TABED_OK;
   RoundArgs& A = h->ra;
-  // QKV, O, gate/up and LM head rows are d_model long and stay whole; only the down projection is cut
-  A.geom[KIND_QKV] = pick_geom(h->qkv_w / 16, h->d, h->d);
-  A.geom[KIND_O] = pick_geom(h->d / 16, h->H * h->hd, h->d);
-  A.geom[KIND_GU] = pick_geom(h->F / 8, h->d, h->d);
-  A.geom[KIND_DN] = pick_geom(h->d / 16, h->F, std::max(h->d, 512));
-  A.geom[KIND_LM] = pick_geom((h->V + 15) / 16, h->d, h->d);
-  int kmax = 0;
+  // d_model is the length of all rows but the down projection's, which is cut; O and down have tiles of 8 rows, as long again
+  A.geom[KIND_QKV] = pick_geom(16, h->qkv_w / 16, h->d, h->d);
+  A.geom[KIND_O] = pick_geom(8, h->d / 8, h->H * h->hd, h->d);
+  A.geom[KIND_GU] = pick_geom(16, h->F / 8, h->d, h->d);
+  A.geom[KIND_DN] = pick_geom(8, h->d / 8, h->F, 2 * std::max(h->d, 256));
+  A.geom[KIND_LM] = pick_geom(16, (h->V + 15) / 16, h->d, h->d);
+  A.slot_bytes = 0;
   long per_step = 0;                                  // upper bound of one CTA's units per decoder step
   for (int k = 0; k < 5; ++k) {
     if (A.geom[k].nsub == 0) return TABED_OK;
-    kmax = std::max(kmax, A.geom[k].kchunk);
+    A.slot_bytes = std::max(A.slot_bytes, A.geom[k].rows * (A.geom[k].kchunk * 2 + 16));
     per_step += (long)((A.geom[k].n_tiles + n_cta - 1) / n_cta) * A.geom[k].nsub * (k == KIND_LM ? 1 : h->L);
   }
   if (per_step > kMaxUnits) return TABED_OK;
   {
-    // the staging of a whole input row: its warps keep at most 8 pieces of 16 bytes per lane in flight
-    const int act_slots = prepass ? h->R : 2 * h->R, warps_per_row = kPW / act_slots;
-    if ((h->d / 2 + warps_per_row * 32 - 1) / (warps_per_row * 32) > 8) return TABED_OK;
+    // wider steps of many rows stay where they were measured
+    const int slots = prepass ? h->R : 2 * h->R;
+    if (h->d > 512 * (16 / slots)) return TABED_OK;
   }
-  A.slot_bytes = 16 * (kmax * 2 + 16);
-  A.act_slots = prepass ? h->R : 2 * h->R;
   A.prepass = prepass ? 1 : 0;
-  const int dn_areas = std::min(A.geom[KIND_DN].nsub, kWG);
-  const size_t act_raw = std::max((size_t)A.act_slots * (h->d + 8) * 2, (size_t)dn_areas * A.act_slots * (A.geom[KIND_DN].kchunk + 8) * 2);
-  A.act_bytes = (int)((act_raw + 127) / 128 * 128);
-  const size_t u_bytes = std::max<size_t>((size_t)A.act_bytes + 2 * kPW * 128 * sizeof(float), (size_t)kPW * 512 * sizeof(float));
+  const size_t u_bytes = ((size_t)kPPartFloats + (size_t)kGW * grp * h->hd) * sizeof(float);
   const size_t avail = (size_t)prop.sharedMemPerBlockOptin - fa.sharedSizeBytes - 1024;
-  if (avail < u_bytes + (size_t)kWG * A.slot_bytes) return TABED_OK;      // a round needs kWG units in flight
-  A.n_ring = (int)std::min<size_t>(kPRing, (avail - u_bytes) / A.slot_bytes);
-  h->persist_smem = (size_t)A.n_ring * A.slot_bytes + u_bytes;
+  // chunks of K and V on their way: as many as a CTA may have to walk through one behind the other, as long as the weights'
+  // ring keeps more than a round's units
+  const size_t kv_bytes = (size_t)kGT * h->hd * 2, per_cta = ((size_t)2 * h->R * h->Hkv * ((h->cap + kPPos - 1) / kPPos) + n_cta - 1) / n_cta;
+  A.kv_stages = 1;
+  while (A.kv_stages < kPMaxStages && (size_t)A.kv_stages < per_cta && u_bytes + (A.kv_stages + 1) * kv_bytes + (size_t)(kPRound + 1) * A.slot_bytes <= avail) ++A.kv_stages;
+  const size_t fixed_bytes = u_bytes + A.kv_stages * kv_bytes;
+  if (avail < fixed_bytes + 3 * (size_t)A.slot_bytes) return TABED_OK;
+  A.n_ring = (int)std::min<size_t>(kPRing, (avail - fixed_bytes) / A.slot_bytes);
+  A.round_units = std::min(kPRound, A.n_ring);
+  h->persist_smem = (size_t)A.n_ring * A.slot_bytes + fixed_bytes;
   // (the device's opt-in maximum, not this handle's own size: a later handle with a smaller ring must not lower it)
   const int persist_attr = (int)((size_t)prop.sharedMemPerBlockOptin - fa.sharedSizeBytes);
-  if (cudaFuncSetAttribute(k_draft_round<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, persist_attr) != cudaSuccess ||
-      cudaFuncSetAttribute(k_draft_round<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, persist_attr) != cudaSuccess)
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, persist_attr) != cudaSuccess ||
+      cudaFuncSetAttribute(kern_trace, cudaFuncAttributeMaxDynamicSharedMemorySize, persist_attr) != cudaSuccess)
     return TABED_ERR_CUDA;
   int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_draft_round<true>, kPT, h->persist_smem) != cudaSuccess) return TABED_ERR_CUDA;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern_trace, kPT, h->persist_smem) != cudaSuccess) return TABED_ERR_CUDA;
   if (per_sm < 1) return TABED_OK;
   h->n_cta = n_cta;
 
@@ -522,15 +534,16 @@ int setup_persistent(tabed_handle* h) {
     if (rc == TABED_OK) rc = dev_alloc(h, ptr, count);           // zeroed: no launch ever stamps epoch 0
     if (rc == TABED_OK) h->ll_all.push_back({*ptr, std::max<size_t>(count, 1) * sizeof(uint2)});
   };
-  LL(&h->ll_xa, kPSlots * d); LL(&h->ll_x1, kPSlots * d); LL(&h->ll_qkv, (size_t)kPSlots * h->qkv_w);
-  LL(&h->ll_mid, (size_t)kPSlots * h->F / 2);
-  LL(&h->ll_po, (size_t)kPSlots * h->H * h->max_splits * h->hd); LL(&h->ll_pml, (size_t)kPSlots * h->H * h->max_splits * 2);
-  LL(&h->ll_rowmax, (size_t)n_cta * kPSlots); LL(&h->ll_rowmax2, (size_t)n_cta * kPSlots); LL(&h->ll_rowsum, (size_t)n_cta * kPSlots * 2);
-  LL(&h->ll_cmass, (size_t)h->B * h->n_chunks * 2); LL(&h->ll_probe, 2);
+  LL(&h->ll_xa, kPSlots * d); LL(&h->ll_x1, kPSlots * d); LL(&h->ll_qkv, (size_t)kPSlots * h->qkv_w / 2);
+  LL(&h->ll_att, kPSlots * d / 2); LL(&h->ll_mid, (size_t)kPSlots * h->F / 2);
+  A.n_part = std::min((h->cap + kPPos - 1) / kPPos, n_cta + 1);      // (a pair has at most one segment per CTA)
+  LL(&h->ll_part, (size_t)kPSlots * h->H * A.n_part * h->hd * 4);
+  LL(&h->ll_rowmax, (size_t)(n_cta + 1) * kPSlots); LL(&h->ll_rowsum, (size_t)n_cta * kPSlots * 2);
+  LL(&h->ll_slice, (size_t)h->B * n_cta * 2); LL(&h->ll_mass, (size_t)h->B * h->V * 2); LL(&h->ll_probe, 2);
   // private copy of the weights, unit by unit (one contiguous block per bulk copy)
   size_t unit_bytes[5], kind_bytes[5];
   for (int k = 0; k < 5; ++k) {
-    unit_bytes[k] = 16 * ((size_t)A.geom[k].kchunk * 2 + 16);
+    unit_bytes[k] = A.geom[k].rows * ((size_t)A.geom[k].kchunk * 2 + 16);
     kind_bytes[k] = unit_bytes[k] * A.geom[k].n_units;
   }
   A.pack_off[KIND_QKV] = 0;
@@ -545,6 +558,36 @@ int setup_persistent(tabed_handle* h) {
     h->allocs.push_back(ptr);
     h->packed = reinterpret_cast<unsigned char*>(ptr);
   }
+  // every CTA's units of a decoder step: the tiles of a phase are dealt round-robin over the CTAs, starting where the phase
+  // before stopped, so that every CTA streams about the same number of bytes; the LM head's in contiguous ranges, which make a
+  // CTA's slice of the vocabulary
+  const int n_phase = 4 * h->L + 1;
+  std::vector<std::vector<uint32_t>> units(n_cta);
+  std::vector<uint16_t> pstart((size_t)n_cta * (n_phase + 1));
+  int next = 0;
+  for (int p = 0; p <= n_phase; ++p) {
+    for (int c = 0; c < n_cta; ++c) pstart[(size_t)c * (n_phase + 1) + p] = (uint16_t)units[c].size();
+    if (p == n_phase) break;
+    const int kind = p == n_phase - 1 ? KIND_LM : (p & 3), nt = A.geom[kind].n_tiles;
+    if (kind == KIND_LM) {
+      for (int c = 0; c < n_cta; ++c)
+        for (int t = (int)((long long)c * nt / n_cta); t < (int)((long long)(c + 1) * nt / n_cta); ++t) units[c].push_back(unit_pack(kind, p >> 2, t, 0));
+      continue;
+    }
+    for (int t = 0; t < nt; ++t, next = (next + 1) % n_cta)
+      for (int sub = 0; sub < A.geom[kind].nsub; ++sub) units[next].push_back(unit_pack(kind, p >> 2, t, sub));
+  }
+  A.max_units = 0;
+  for (const auto& u : units) A.max_units = std::max(A.max_units, (int)u.size());
+  std::vector<uint32_t> ulist((size_t)n_cta * A.max_units);
+  for (int c = 0; c < n_cta; ++c) std::copy(units[c].begin(), units[c].end(), ulist.begin() + (size_t)c * A.max_units);
+  uint16_t* d_pstart = nullptr;
+  uint32_t* d_ulist = nullptr;
+  A2(&d_pstart, pstart.size()); A2(&d_ulist, ulist.size());
+  if (rc == TABED_OK && (cudaMemcpyAsync(d_pstart, pstart.data(), pstart.size() * sizeof(uint16_t), cudaMemcpyHostToDevice, h->stream) != cudaSuccess ||
+                         cudaMemcpyAsync(d_ulist, ulist.data(), ulist.size() * sizeof(uint32_t), cudaMemcpyHostToDevice, h->stream) != cudaSuccess))
+    rc = TABED_ERR_CUDA;
+  A.pstart = d_pstart; A.ulist = d_ulist;
   h->trace_stride = 5 * h->L + 8;
   A2(&h->trace, (size_t)h->G * h->trace_stride * kTraceRec);
   if (rc != TABED_OK) return rc;
@@ -560,7 +603,7 @@ int setup_persistent(tabed_handle* h) {
     for (int k = 0; k < 5; ++k) {
       if ((l == h->L) != (k == KIND_LM)) continue;
       PackArgs P{};
-      P.kind = k; P.g = A.geom[k];
+      P.kind = k; P.g = A.geom[k]; P.hd = h->hd;
       P.dst = h->packed + A.pack_off[k] + (k == KIND_LM ? 0 : (size_t)l * A.pack_layer_stride);
       if (k == KIND_QKV) { P.w0 = tab[l].wq; P.w1 = tab[l].wk; P.w2 = tab[l].wv; P.rows0 = h->d; P.rows1 = kvd; P.rows2 = kvd; P.K = h->d; }
       else if (k == KIND_O) { P.w0 = tab[l].wo; P.rows0 = h->d; P.K = h->H * h->hd; }
@@ -577,11 +620,10 @@ int setup_persistent(tabed_handle* h) {
   A.eps = c.rms_eps; A.attn_scale = 1.0f / sqrtf((float)h->hd);
   A.R = h->R; A.B = h->B; A.m = h->m; A.G = h->G; A.greedy = c.sample_mode == TABED_MODE_GREEDY;
   A.kv_len = h->kv_len; A.pending = h->pending; A.kc = (bf*)h->kc; A.vc = (bf*)h->vc;
-  A.xa = h->ll_xa; A.x1 = h->ll_x1; A.qkv = h->ll_qkv; A.mid = h->ll_mid;
-  A.part_o = h->ll_po; A.part_ml = h->ll_pml; A.max_splits = h->max_splits;
+  A.xa = h->ll_xa; A.x1 = h->ll_x1; A.qkv = h->ll_qkv; A.att = h->ll_att; A.mid = h->ll_mid; A.part = h->ll_part;
   A.logits_own = h->logits_own; A.w = h->w; A.qk = h->qk; A.q = h->q;
-  A.rowmax = h->ll_rowmax; A.rowmax2 = h->ll_rowmax2; A.rowsum = h->ll_rowsum; A.chunk_mass = h->ll_cmass;
-  A.n_chunks = h->n_chunks; A.tokens = h->tokens; A.err = h->err; A.packed = h->packed;
+  A.rowmax = h->ll_rowmax; A.rowsum = h->ll_rowsum; A.slice_mass = h->ll_slice; A.mass = h->ll_mass;
+  A.tokens = h->tokens; A.err = h->err; A.packed = h->packed;
   A.trace_stride = h->trace_stride;
   h->persist_ok = true;
   return TABED_OK;
@@ -591,7 +633,6 @@ int launch_persistent_round(tabed_handle* h, const float* u_draft, int32_t* out_
   RoundArgs A = h->ra;
   A.u = u_draft; A.out_tokens = out_tokens; A.logits_override = h->logits_override;
   (void)max_pos;
-  A.split_len = (h->hd <= 64) ? 256 : 128;          // positions per attention item: 4 register passes of the CTA
   // epochs: this launch stamps epoch0 + 1 ... epoch0 + (G [+ 1]) (5 L + 8); when the counter nears its end the buffers are cleared
   const unsigned span = (unsigned)(h->G + (A.prepass ? 1 : 0)) * (5u * (unsigned)h->L + 8u);
   if (h->ll_epoch > 0xFFFFFFFFu - 2u * span) {
@@ -602,8 +643,7 @@ int launch_persistent_round(tabed_handle* h, const float* u_draft, int32_t* out_
   h->ll_epoch += span;
   A.trace = h->trace_on ? h->trace : nullptr; A.trace_cta = h->trace_cta;
   void* args[] = {&A};
-  const void* kern = h->trace_on ? (const void*)k_draft_round<true> : (const void*)k_draft_round<false>;
-  if (cudaLaunchCooperativeKernel(kern, dim3(h->n_cta), dim3(kPT), args, h->persist_smem, h->stream) != cudaSuccess)
+  if (cudaLaunchCooperativeKernel(draft_round_kernel(h, h->trace_on), dim3(h->n_cta), dim3(kPT), args, h->persist_smem, h->stream) != cudaSuccess)
     return TABED_ERR_CUDA;
   h->launches_persist++;
   h->launches++;
@@ -1396,10 +1436,8 @@ namespace {
 // One CTA polls a flagged word for an epoch that nobody writes: the bounded wait runs out, the error bit is set
 // and the kernel returns.
 __global__ void __launch_bounds__(kPT) k_wait_probe(const uint2* word, int* err) {
-  __shared__ PShared S;
-  if (threadIdx.x == 0) S.dead = 0;
-  __syncthreads();
-  if (threadIdx.x == 0) ll_wait1(word, 0xFFFFFFFFu, S, err);
+  int dead = 0;
+  if (threadIdx.x == 0) ll_wait1(word, 0xFFFFFFFFu, dead, err);
   __syncthreads();
 }
 }  // namespace
