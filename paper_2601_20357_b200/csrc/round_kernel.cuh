@@ -405,12 +405,14 @@ __device__ __forceinline__ uint4 ll_wait2(const uint2* p, uint32_t epoch, int& d
 }
 
 // A lane's pieces of K and V of chunk c (of n) in a layer, into its places of a stage: one group of copies, empty where there is
-// no such chunk or no cached position for the warp.  A lane without a position of its own asks for the last one (a weight of 0
+// no such chunk or no cached position for the warp.  (16 bytes each, which go past the L1: it does not see the rows that other
+// SMs append.)  A lane without a position of its own asks for the last one (a weight of 0
 // does not cancel what an unwritten row may hold).
+template <int HD> __host__ __device__ constexpr int kv_pieces() { return HD == 32 ? 6 : HD / 8; }      // of K and V, per lane
 template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 template <int HD>
 __device__ __forceinline__ void kv_request(const RoundArgs& A, PShared& S, unsigned char* stage, int c, int n, int layer, int gw, int lane) {
-  constexpr int KP = HD / 32, VP = HD / 64, kPiece = kGT * 16;
+  constexpr int KP = HD / 32, VP = HD <= 64 ? 1 : HD / 64, kPiece = kGT * 16;
   if (c < n) {
     const uint32_t e = uni(S.chunks[c]);
     const int s = e & 7, gk = (e >> 3) & 63, split = (e >> 9) & 511, gq = lane >> 2, t4 = lane & 3;
@@ -427,14 +429,9 @@ __device__ __forceinline__ void kv_request(const RoundArgs& A, PShared& S, unsig
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         const __nv_bfloat16* src = A.vc + (size_t)(row + min((i >> 1) * 8 + 2 * t4 + (i & 1), lim - 1)) * HD;
-        if constexpr (HD == 32) {                              // half a piece: dims 8 (g & 3) + 4 (g >> 2) ..
-          asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst + (i & 1) * 8), "l"(src + (gq & 3) * 8 + (gq >> 2) * 4) : "memory");
-          if (i & 1) dst += kPiece;
-        } else {
 #pragma unroll
-          for (int j = 0; j < VP; ++j, dst += kPiece)          // pieces g, g + 8
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src + (gq + 8 * j) * 8) : "memory");
-        }
+        for (int j = 0; j < VP; ++j, dst += kPiece)            // pieces g, g + 8 (head size 32: g & 3, of which the lane uses half)
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src + ((HD == 32 ? gq & 3 : gq) + 8 * j) * 8) : "memory");
       }
     }
   }
@@ -540,7 +537,7 @@ __global__ void __launch_bounds__(kPT, 1) k_draft_round(const RoundArgs A) {
   float* s_o = part + kPPartFloats;                      // attention: [kGW][grp * HD]
   const int kvd = A.Hkv * HD, grp = A.H / A.Hkv;
   // K and V on their way: kv_stages times [piece][warp of group 1][lane][16 bytes]
-  constexpr int kv_piece = kGT * 16, kv_stage_bytes = HD / 8 * kv_piece;
+  constexpr int kv_piece = kGT * 16, kv_stage_bytes = kv_pieces<HD>() * kv_piece;
   unsigned char* kv_area = reinterpret_cast<unsigned char*>(s_o + kGW * grp * HD);
   constexpr int half = HD >> 1;
   const int R = A.R, B = A.B, m = A.m, G = A.G, V = A.V, d = A.d;
@@ -911,7 +908,7 @@ __global__ void __launch_bounds__(kPT, 1) k_draft_round(const RoundArgs A) {
             // the positions produced in this very phase come as words: they take their places in the stage, the last one in the cache too
             if (cached <= 0) {                                 // (nothing was asked for: the places of the others must not hold what is not finite)
 #pragma unroll
-              for (int i = 0; i < HD / 8; ++i) *reinterpret_cast<uint4*>(st + i * kv_piece) = make_uint4(0u, 0u, 0u, 0u);
+              for (int i = 0; i < kv_pieces<HD>(); ++i) *reinterpret_cast<uint4*>(st + i * kv_piece) = make_uint4(0u, 0u, 0u, 0u);
             }
 #pragma unroll 1
             for (int j = 0; j < n_fresh; ++j) {
@@ -948,7 +945,7 @@ __global__ void __launch_bounds__(kPT, 1) k_draft_round(const RoundArgs A) {
                 const int i = (r >> 3) * 2 + (r & 1);
                 if constexpr (HD == 32) {
                   const uint2 v4 = make_uint2(x[2 * KP].x, x[2 * KP].z);
-                  *reinterpret_cast<uint2*>(st + (2 * KP + (i >> 1)) * kv_piece + (i & 1) * 8) = v4;
+                  *reinterpret_cast<uint2*>(st + (2 * KP + i) * kv_piece + (gq >> 2) * 8) = v4;
                   if (j == 0) *reinterpret_cast<uint2*>(A.vc + row + (gq & 3) * 8 + (gq >> 2) * 4) = v4;
                 } else {
 #pragma unroll
@@ -967,7 +964,7 @@ __global__ void __launch_bounds__(kPT, 1) k_draft_round(const RoundArgs A) {
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
               if constexpr (HD == 32) {
-                const uint2 x = *reinterpret_cast<const uint2*>(st + (2 * KP + (i >> 1)) * kv_piece + (i & 1) * 8);
+                const uint2 x = *reinterpret_cast<const uint2*>(st + (2 * KP + i) * kv_piece + (gq >> 2) * 8);     // dims 8 (g & 3) + 4 (g >> 2) ..
                 vw[i][0] = x.x; vw[i][1] = x.y;
               } else {
 #pragma unroll

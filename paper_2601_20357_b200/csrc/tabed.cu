@@ -508,7 +508,7 @@ int setup_persistent(tabed_handle* h) {
   const size_t avail = (size_t)prop.sharedMemPerBlockOptin - fa.sharedSizeBytes - 1024;
   // chunks of K and V on their way: as many as a CTA may have to walk through one behind the other, as long as the weights'
   // ring keeps more than a round's units
-  const size_t kv_bytes = (size_t)kGT * h->hd * 2, per_cta = ((size_t)2 * h->R * h->Hkv * ((h->cap + kPPos - 1) / kPPos) + n_cta - 1) / n_cta;
+  const size_t kv_bytes = (size_t)kGT * 16 * (h->hd == 32 ? kv_pieces<32>() : (h->hd == 64 ? kv_pieces<64>() : kv_pieces<128>())), per_cta = ((size_t)2 * h->R * h->Hkv * ((h->cap + kPPos - 1) / kPPos) + n_cta - 1) / n_cta;
   A.kv_stages = 1;
   while (A.kv_stages < kPMaxStages && (size_t)A.kv_stages < per_cta && u_bytes + (A.kv_stages + 1) * kv_bytes + (size_t)(kPRound + 1) * A.slot_bytes <= avail) ++A.kv_stages;
   const size_t fixed_bytes = u_bytes + A.kv_stages * kv_bytes;
