@@ -278,10 +278,10 @@ int tabed_last_device_error(tabed_handle* h);
  * by itself.  Errors: BAD_STATE (mid-round), CUDA. */
 int tabed_sync_lengths(tabed_handle* h);
 
-/* Test aid for the failure path of the device-side waits: launches ONE CTA that waits, with the persistent
- * kernel's own bounded poll, for a flagged word that nobody writes, so that the wait (about 2^21 polls, a
- * fraction of a second) runs out, records the failure and returns by itself - the GPU keeps
- * answering.  Returns what tabed_last_device_error then reports (TABED_ERR_TIMEOUT).
+/* Test aid for the failure path of the device-side waits: launches ONE CTA that waits, with each of the persistent
+ * kernel's own bounded waits, for words and a copy that nobody sends, so that every wait (about 2^21 polls, a
+ * second or two) runs out, records the failure and returns by itself - the GPU keeps
+ * answering.  Returns what tabed_last_device_error then reports (TABED_ERR_TIMEOUT; OK if a wait did not run out).
  * Errors: UNSUPPORTED (handle without the persistent kernel), CUDA. */
 int tabed_debug_barrier_timeout(tabed_handle* h);
 

@@ -64,6 +64,7 @@ constexpr int kMaxUnits = 1024;          // units of one CTA in one decoder step
 constexpr int kMaxPhase = 4 * kPMaxL + 1;
 constexpr int kPMaxChunks = 1280;        // attention chunks of one CTA
 constexpr int kPMaxStages = 3;           // chunks of K and V on their way to a warp
+constexpr int kProbeWords = 128;         // words that nobody writes, for the test of the bounded waits (64 masses of two words)
 // Partial tiles of a round in shared memory: [unit][slot pair][warp][2][16 rows], 40 floats a warp and 8 idle ones a pair, which
 // make the fragments' stores and the sums' loads free of bank conflicts.  Up to 4 slots take two pairs and rounds of 4 units,
 // up to 8 slots four pairs and rounds of 2 units; two buffers a group, so that a round needs one barrier; group 1 has one tile
@@ -382,6 +383,8 @@ __device__ __forceinline__ void ll_poll(const uint2* p, int n, uint32_t epoch, u
 #pragma unroll
     for (int j = 0; j < N; ++j) miss |= (v[j].y ^ epoch) | (v[j].w ^ epoch);
     if (!__any_sync(0xffffffffu, miss != 0 && !dead)) break;
+    // (a lane may come in with a wait of its own that ran out: the warp stays together, or the votes below would miss it)
+    if (__any_sync(0xffffffffu, dead)) { dead = 1; break; }
     uint4 x;
 #pragma unroll 1
     do {

@@ -100,7 +100,7 @@ struct tabed_handle {
   uint2 *ll_rowmax = nullptr, *ll_rowsum = nullptr, *ll_slice = nullptr, *ll_mass = nullptr;
   std::vector<std::pair<void*, size_t>> ll_all;       // every exchange buffer (cleared when the epoch counter wraps)
   unsigned ll_epoch = 0;
-  uint2* ll_probe = nullptr;        // a word nobody ever writes (tabed_debug_barrier_timeout)
+  uint2* ll_probe = nullptr;        // words nobody ever writes (tabed_debug_barrier_timeout)
   // tensor-core streaming attention of the per-operation paths (bf16 caches, head size 64)
   int* attn_tickets = nullptr; int n_sm = 0;
   bool atc_ok = false; CUtensorMap tm_k, tm_v;
@@ -539,7 +539,7 @@ int setup_persistent(tabed_handle* h) {
   A.n_part = std::min((h->cap + kPPos - 1) / kPPos, n_cta + 1);      // (a pair has at most one segment per CTA)
   LL(&h->ll_part, (size_t)kPSlots * h->H * A.n_part * h->hd * 4);
   LL(&h->ll_rowmax, (size_t)(n_cta + 1) * kPSlots); LL(&h->ll_rowsum, (size_t)n_cta * kPSlots * 2);
-  LL(&h->ll_slice, (size_t)h->B * n_cta * 2); LL(&h->ll_mass, (size_t)h->B * h->V * 2); LL(&h->ll_probe, 2);
+  LL(&h->ll_slice, (size_t)h->B * n_cta * 2); LL(&h->ll_mass, (size_t)h->B * h->V * 2); LL(&h->ll_probe, kProbeWords);
   // private copy of the weights, unit by unit (one contiguous block per bulk copy)
   size_t unit_bytes[5], kind_bytes[5];
   for (int k = 0; k < 5; ++k) {
@@ -1433,12 +1433,28 @@ int tabed_round_host(tabed_handle* h, const float* u_draft, const float* u_accep
 }
 
 namespace {
-// One CTA polls a flagged word for an epoch that nobody writes: the bounded wait runs out, the error bit is set
-// and the kernel returns.
-__global__ void __launch_bounds__(kPT) k_wait_probe(const uint2* word, int* err) {
-  int dead = 0;
-  if (threadIdx.x == 0) ll_wait1(word, 0xFFFFFFFFu, dead, err);
+// One CTA, a warp for each kind of wait: on words and a copy that nobody sends, every wait runs out by itself.  The error bits
+// are handed on only if each warp came back from its wait with its timeout.
+__global__ void __launch_bounds__(kPT) k_wait_probe(const uint2* words, int* err) {
+  __shared__ PShared S;
+  __shared__ int n_out, bits;
+  const unsigned epoch = 0xFFFFFFFFu;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) { n_out = bits = 0; S.issued[0] = 0; mbar_init(&S.full[0], 1); }
   __syncthreads();
+  int dead = 0;
+  uint4 v[4];
+  if (warp == 0) ll_poll<4, 2, 16>(words, 2, epoch, v, dead, &bits);
+  // (a lane's own wait has run out, the others' have not: the warp's next poll takes it back whole)
+  if (warp == 1 && lane == 5) ll_wait1(words, epoch, dead, &bits);
+  __syncwarp();
+  if (warp == 1) ll_poll<4, 2, 16>(words, 2, epoch, v, dead, &bits);
+  if (warp == 2) ll_wait2(words + 2 * lane, epoch, dead, &bits);
+  if (warp == 3) dead = find_mass(words, kProbeWords / 2, true, 0.5f, epoch, 0ull, dead, &bits).dead;
+  if (warp == 4) wait_full(S, 0, 0, dead, &bits);
+  if (__all_sync(0xffffffffu, dead) && lane == 0) atomicAdd(&n_out, 1);
+  __syncthreads();
+  if (threadIdx.x == 0 && n_out == 5) atomicOr(err, bits);
 }
 }  // namespace
 

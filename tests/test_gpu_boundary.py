@@ -60,7 +60,8 @@ def test_a_bounded_wait_that_runs_out_is_reported_and_the_gpu_keeps_answering():
     pair = H.build_pair(small_wl(cid=71))
     g = pair.gpu
     assert g.current_path() == TB.PATH_PERSISTENT
-    assert g.debug_barrier_timeout() == TB.ERR_TIMEOUT    # one CTA, an arrival count nobody completes: the wait gives up
+    # one CTA, a warp for each kind of wait (one of them comes in with a lane whose own wait has run out): all give up
+    assert g.debug_barrier_timeout() == TB.ERR_TIMEOUT
     assert g.last_device_error() == 0
     for rnd in range(2):                                  # the persistent kernel's own barriers are intact afterwards
         H.lockstep_round(pair, rnd, override=True)
