@@ -862,7 +862,7 @@ __global__ void __launch_bounds__(kPT, 1) k_draft_round(const RoundArgs A) {
       // The caches of all (slot, KV head) pairs are cut into chunks of kPPos positions; the chunks, in (slot, head,
       // position) order, are dealt to the CTAs in contiguous ranges, so a CTA walks along one cache for several chunks.
       // A warp owns 16 positions of a chunk: K and V as mma A fragments (positions, resp. dims, as rows; the heads of the group
-      // are the 8 columns of B): scores^T = K q^T, out^T = V^T P^T with P as bf16 head + remainder.
+      // are the 8 columns of B): scores^T = K q^T, out^T = V^T P^T with P as a sum of bf16 terms.
       // The order of the summed index of a product is free, so the dims of q.k are dealt to the k-steps such that lane (g, t)
       // needs whole 16-byte pieces t, t + 4 ... of rows g and g + 8; in V^T P^T rows g and g + 8 of an m-tile stand for two
       // neighbouring dims of the pieces that the lane holds of the four positions 2t, 2t+1, 8+2t, 9+2t (pairs of
@@ -995,31 +995,54 @@ __global__ void __launch_bounds__(kPT, 1) k_draft_round(const RoundArgs A) {
             float pw[4];
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
-              const float s0 = gq < lim ? (sc[0][e] + sc[1][e]) * scale2 : -INFINITY, s1 = gq + 8 < lim ? (sc[0][e + 2] + sc[1][e + 2]) * scale2 : -INFINITY;
-              float mx = fmaxf(s0, s1);
+              // (the maximum is of the rounded products, any reference will do; the weight's exponent is rounded once, behind the
+              // subtraction: a score's own rounding would cost a weight 2^-24 times the score)
+              const float x0 = gq < lim ? sc[0][e] + sc[1][e] : -INFINITY, x1 = gq + 8 < lim ? sc[0][e + 2] + sc[1][e + 2] : -INFINITY;
+              float mx = fmaxf(x0 * scale2, x1 * scale2);
 #pragma unroll
               for (int o = 4; o < 32; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(FULL, mx, o));
               const float Mn = fmaxf(m_run[e], mx), N = Mn > -INFINITY ? Mn : 0.0f, f = ex2_approx(m_run[e] - N);
               m_run[e] = Mn;
-              pw[e] = ex2_approx(s0 - N); pw[e + 2] = ex2_approx(s1 - N);
+              pw[e] = ex2_approx(fmaf(x0, scale2, -N)); pw[e + 2] = ex2_approx(fmaf(x1, scale2, -N));
               l_run[e] = fmaf(l_run[e], f, pw[e] + pw[e + 2]);
 #pragma unroll
               for (int j = 0; j < MT; ++j) { oc[j][e] *= f; oc[j][e + 2] *= f; }
             }
-            // the weights as a bf16 head and a bf16 remainder (two products, fp32 sums), moved from accumulator layout
-            // (positions as rows) to B-operand layout (positions as the summed index)
-            uint32_t wh[2], wl[2];
-            {
-              const float h0 = round_bf16(pw[0]), h1 = round_bf16(pw[1]), h2 = round_bf16(pw[2]), h3 = round_bf16(pw[3]);
-              wh[0] = movmatrix_trans(pack_bf16(h0, h1)); wh[1] = movmatrix_trans(pack_bf16(h2, h3));
-              wl[0] = movmatrix_trans(pack_bf16(pw[0] - h0, pw[1] - h1)); wl[1] = movmatrix_trans(pack_bf16(pw[2] - h2, pw[3] - h3));
-            }
+            // The weights as bf16 terms of 8 bits (fp32 sums), moved from accumulator layout (positions as rows) to B-operand
+            // layout (positions as the summed index): three terms, all of an fp32 weight - two for the cached positions of head size 64.
+            // (With two for all of them a sum of 300 positions that cancel is eleven times as far off, at head sizes 32 and 128; the
+            // third costs 2 - 3 % of a round over 6000 positions there, and at head size 64, for the new positions, 1 % at 8192.)
+            uint32_t t0, t1, w0[2], w1[2], w2[2];
+            auto term = [&](uint32_t (&w)[2]) {
+              t0 = pack_bf16(pw[0], pw[1]); t1 = pack_bf16(pw[2], pw[3]);
+              w[0] = movmatrix_trans(t0); w[1] = movmatrix_trans(t1);
+            };
+            auto remainder = [&]() {
+              pw[0] -= __uint_as_float(t0 << 16); pw[1] -= __uint_as_float(t0 & 0xFFFF0000u);
+              pw[2] -= __uint_as_float(t1 << 16); pw[3] -= __uint_as_float(t1 & 0xFFFF0000u);
+            };
+            auto values = [&](int j, uint32_t (&af)[4]) {
+              af[0] = __byte_perm(vw[0][j], vw[1][j], 0x5410u); af[1] = __byte_perm(vw[0][j], vw[1][j], 0x7632u);
+              af[2] = __byte_perm(vw[2][j], vw[3][j], 0x5410u); af[3] = __byte_perm(vw[2][j], vw[3][j], 0x7632u);
+            };
+            term(w0); remainder(); term(w1);
+            if constexpr (HD != 64) { remainder(); term(w2); }
 #pragma unroll
             for (int j = 0; j < MT; ++j) {
-              const uint32_t af[4] = {__byte_perm(vw[0][j], vw[1][j], 0x5410u), __byte_perm(vw[0][j], vw[1][j], 0x7632u),
-                                      __byte_perm(vw[2][j], vw[3][j], 0x5410u), __byte_perm(vw[2][j], vw[3][j], 0x7632u)};
-              mma_bf16(oc[j], af, wh);
-              mma_bf16(oc[j], af, wl);
+              uint32_t af[4];
+              values(j, af);
+              mma_bf16(oc[j], af, w0);
+              mma_bf16(oc[j], af, w1);
+              if constexpr (HD != 64) mma_bf16(oc[j], af, w2);
+            }
+            if (HD == 64 && cached < 16) {
+              remainder(); term(w2);
+#pragma unroll
+              for (int j = 0; j < MT; ++j) {
+                uint32_t af[4];
+                values(j, af);
+                mma_bf16(oc[j], af, w2);
+              }
             }
           }
           if (split == nsplit - 1 || gc == n_chunk - 1) {
@@ -1079,13 +1102,18 @@ __global__ void __launch_bounds__(kPT, 1) k_draft_round(const RoundArgs A) {
             uint4 raw[12];
             const int n = min(6, n_seg - j0);
             ll_poll<12, 2, HD * 4>(p, n, ep_att, raw, dead, A.err);
+            float Mn = M;
+#pragma unroll
+            for (int j = 0; j < 6; ++j) if (j < n) Mn = fmaxf(Mn, __uint_as_float(raw[2 * j].z));
+            const float N = Mn > -INFINITY ? Mn : 0.0f, fo = ex2_approx(M - N);
+            v *= fo; l *= fo;
 #pragma unroll
             for (int j = 0; j < 6; ++j) {
               if (j >= n) break;
-              const float mq = __uint_as_float(raw[2 * j].z), Mn = fmaxf(M, mq), N = Mn > -INFINITY ? Mn : 0.0f, fo = ex2_approx(M - N), f = ex2_approx(mq - N);
-              v = fmaf(f, __uint_as_float(raw[2 * j].x), v * fo); l = fmaf(f, __uint_as_float(raw[2 * j + 1].x), l * fo);
-              M = Mn;
+              const float f = ex2_approx(__uint_as_float(raw[2 * j].z) - N);
+              v = fmaf(f, __uint_as_float(raw[2 * j].x), v); l = fmaf(f, __uint_as_float(raw[2 * j + 1].x), l);
             }
+            M = Mn;
           }
           store_att(A, ps, head * HD + dd, v / l, ep_att);
         }

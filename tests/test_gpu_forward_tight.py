@@ -134,3 +134,61 @@ def test_one_step_on_identical_caches(name, path):
         assert x <= max(3.0 * o, f), f"{what} {x:.3e} above 3 x {o:.1e}"
     assert dprob <= H.PROB_TOL
     g.destroy()
+
+
+@pytest.mark.parametrize("hd", [32, 128])
+def test_attention_weights_carry_fp32(hd):
+    """Softmax weights and exponentials of the persistent kernel's attention at fp32's precision, where they always had it.
+
+    One layer whose only work is the attention: the residual is a row of +-1 (its norm is 1, so q is free of ties), the values
+    of the new position and the feed-forward part are zero, the output projection is c times the identity and the LM head is the
+    identity, so the logits are (x + c o) / rms.  The last cached values are chosen (bf16 each, one behind the other) so that
+    the exact attention output o is zero: what is left of it is the error of the weights.  If each weight is off by an independent
+    2^-22 of itself (fp32's exponential and its argument), the error of o is 2^-22 sqrt(sum (w v)^2); weights of 16 bits give
+    2^-18 / sqrt 3, nine times that.  c makes the former 1/4 of the residual; the logits' own bf16 rounding adds 2^-9."""
+    heads, n = 256 // hd, 300
+    d = heads * hd
+    cfg = W.DrafterCfg(1, d, heads, heads, 16, d, "bf16")
+    wl = W.Workload(name=f"weights{hd}", config_id=57, drafter=cfg, n_inputs=1, n_requests=1, gamma=1, window_h=1, rounds=1,
+                    policy=W.POLICY_STATIC, kv_capacity=512)
+    rng = np.random.default_rng(hd)
+    weights = W.make_weights(wl)
+    x = rng.choice([-1.0, 1.0], size=d).astype(np.float32)
+    weights["embed"][:] = x
+    weights["wq"][0] = W.to_bf16_grid(rng.standard_normal((d, d)).astype(np.float32) * np.float32(d ** -0.5))
+    for name in ("wv", "w_down"):
+        weights[name][0] = np.zeros_like(weights[name][0])
+    weights["lm_head"] = np.eye(d, dtype=np.float32)
+    # the weights of the cached positions, from the checker's own q (the first step appends position n)
+    probe = OracleDrafter(cfg, weights)
+    a = probe.rb(probe.rmsnorm(x[None].astype(np.float64), probe.layers[0]["norm1"]))
+    rotated = lambda w: probe.rb(probe.rope((a @ w.T).reshape(1, heads, hd), np.array([n])))[0]
+    q, k_new = rotated(probe.layers[0]["wq"]), rotated(probe.layers[0]["wk"])
+    K = W.to_bf16_grid(rng.standard_normal((heads, n, hd)).astype(np.float32))
+    s = np.einsum("hd,hnd->hn", q, K.astype(np.float64)) / np.sqrt(hd)
+    s_new = (q * k_new).sum(-1, keepdims=True) / np.sqrt(hd)
+    e = np.exp(np.concatenate([s, s_new], 1) - s.max(1, keepdims=True))
+    w = (e / e.sum(1, keepdims=True))[:, :n]
+    V = W.to_bf16_grid(rng.standard_normal((heads, n, hd)).astype(np.float32))
+    order = np.argsort(-w, axis=1)[:, :5]                       # the largest weights take up the sum: coarse first, then fine
+    for h in range(heads):
+        V[h, order[h]] = 0.0
+        for j in order[h]:
+            V[h, j] = W.to_bf16_grid((-(w[h] @ V[h].astype(np.float64)) / w[h, j]).astype(np.float32))
+    rest = np.abs(np.einsum("hn,hnd->hd", w, V.astype(np.float64))).max()
+    unit = np.sqrt(np.mean(np.einsum("hn,hnd->hd", w ** 2, V.astype(np.float64) ** 2)))
+    c = 2.0 ** np.floor(np.log2(0.25 / (2.0 ** -22 * unit)))
+    assert rest * c < 1e-2
+    weights["wo"][0] = (c * np.eye(d)).astype(np.float32)
+    g = H.make_gpu(wl, TB.weights_to_device(cfg, weights, H.DEV))
+    g.load_prefix_kv(0, H.t(K[None], torch.bfloat16), H.t(V[None], torch.bfloat16))
+    g.set_pending(torch.zeros((1, 2), dtype=torch.int32, device=H.DEV), torch.ones(1, dtype=torch.int32, device=H.DEV))
+    assert g.current_path() == TB.PATH_PERSISTENT
+    g.draft_round(torch.full((1, 1), 0.5, device=H.DEV), torch.empty((1, 1), dtype=torch.int32, device=H.DEV))
+    torch.cuda.synchronize()
+    assert g.last_device_error() == 0
+    y = g.debug_view(TB.VIEW_LOGITS).cpu().numpy().reshape(-1).astype(np.float64) * x      # (1 + c o x) / rms
+    err = np.sqrt(np.mean((y / np.mean(y) - 1.0) ** 2))
+    print(f"WEIGHTS hd {hd}: c 2^{int(np.log2(c))}, error of c o {err:.3f}, bound {c * 2.0 ** -22 * unit:.3f}")
+    assert np.mean(y) > 0 and err <= c * 2.0 ** -22 * unit + 2.0 ** -9
+    g.destroy()
