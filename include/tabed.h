@@ -131,7 +131,8 @@ extern "C" {
                                       B*m <= 8 rows (with more than 4 rows at least two layers: the first of
                                       two pending tokens then gets a weight pass of its own), d_model <= 2048
                                       (<= 1024 with more than 4 slots: 3 - 4 or 5 - 8 rows) and
-                                      a multiple of 16, d_ffn a multiple of 16, H <= 64, (H/Hkv)*head_dim <= 512, <= 64 layers,
+                                      a multiple of 16, vocab <= 2^20,
+                                      d_ffn a multiple of 16, H <= 64, (H/Hkv)*head_dim <= 512, <= 64 layers,
                                       kv_capacity <= 32768                                                */
 #define TABED_PATH_TENSOR_CORE 3   /* one kernel per operation with the projections as tcgen05 contractions
                                       over all rows: any bf16 drafter with d_model, d_ffn, H*head_dim

@@ -242,6 +242,7 @@ struct PShared {
 };
 
 // a unit of the list: kind (3 bits), layer (7), sub-unit of its tile (6), tile (16) - no division where it is used
+constexpr int kUnitTiles = 1 << 16;
 __host__ __device__ __forceinline__ uint32_t unit_pack(int kind, int layer, int tile, int sub) {
   return (uint32_t)kind | ((uint32_t)layer << 3) | ((uint32_t)sub << 10) | ((uint32_t)tile << 16);
 }

@@ -493,7 +493,7 @@ int setup_persistent(tabed_handle* h) {
   A.slot_bytes = 0;
   long per_step = 0;                                  // upper bound of one CTA's units per decoder step
   for (int k = 0; k < 5; ++k) {
-    if (A.geom[k].nsub == 0) return TABED_OK;
+    if (A.geom[k].nsub == 0 || A.geom[k].n_tiles > kUnitTiles) return TABED_OK;
     A.slot_bytes = std::max(A.slot_bytes, A.geom[k].rows * (A.geom[k].kchunk * 2 + 16));
     per_step += (long)((A.geom[k].n_tiles + n_cta - 1) / n_cta) * A.geom[k].nsub * (k == KIND_LM ? 1 : h->L);
   }

@@ -58,6 +58,27 @@ def test_path_selection():
     tiny.gpu.destroy()
 
 
+def blank_drafter(cfg):
+    """A handle of one row on weights of zeros (path selection only)."""
+    z = lambda *shape: torch.zeros(shape, dtype=torch.bfloat16, device=H.DEV)
+    d, F, kvd = cfg.d_model, cfg.d_ffn, cfg.n_kv_heads * cfg.head_dim
+    shapes = dict(wq=(d, d), wk=(kvd, d), wv=(kvd, d), wo=(d, d), w_gate=(F, d), w_up=(F, d), w_down=(d, F), norm1=(d,), norm2=(d,))
+    w = {k: [z(*s) for _ in range(cfg.n_layers)] for k, s in shapes.items()}
+    w.update(embed=z(cfg.vocab, d), lm_head=z(cfg.vocab, d), final_norm=z(d))
+    return TB.Tabed(n_inputs=1, n_requests=1, gamma=1, window_h=1, policy=TB.POLICY_STATIC, vocab=cfg.vocab, drafter=cfg, weights=w,
+                    kv_capacity=64)
+
+
+@pytest.mark.parametrize("cfg,persistent", [
+    (W.DrafterCfg(1, 32, 1, 1, 32, 1 << 20, "bf16"), True),             # 65536 LM-head tiles, all that a unit's number holds
+    (W.DrafterCfg(1, 32, 1, 1, 32, (1 << 20) + 1, "bf16"), False),      # one more
+])
+def test_path_selection_at_the_bounds(cfg, persistent):
+    g = blank_drafter(cfg)
+    assert (g.current_path() == TB.PATH_PERSISTENT) == persistent
+    g.destroy()
+
+
 def test_lockstep_gqa_head64_three_inputs():
     """R = 3 slots, grouped-query attention 4/2, one row longer than an attention split (merge by ticket)."""
     run_lockstep(wl_small(), 5).gpu.destroy()
