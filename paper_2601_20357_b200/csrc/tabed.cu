@@ -491,13 +491,34 @@ int setup_persistent(tabed_handle* h) {
   A.geom[KIND_DN] = pick_geom(8, h->d / 8, h->F, 2 * std::max(h->d, 256));
   A.geom[KIND_LM] = pick_geom(16, (h->V + 15) / 16, h->d, h->d);
   A.slot_bytes = 0;
-  long per_step = 0;                                  // upper bound of one CTA's units per decoder step
   for (int k = 0; k < 5; ++k) {
     if (A.geom[k].nsub == 0 || A.geom[k].n_tiles > kUnitTiles) return TABED_OK;
     A.slot_bytes = std::max(A.slot_bytes, A.geom[k].rows * (A.geom[k].kchunk * 2 + 16));
-    per_step += (long)((A.geom[k].n_tiles + n_cta - 1) / n_cta) * A.geom[k].nsub * (k == KIND_LM ? 1 : h->L);
   }
-  if (per_step > kMaxUnits) return TABED_OK;
+  // every CTA's units of a decoder step: the tiles of a phase are dealt round-robin over the CTAs, starting where the phase
+  // before stopped, so that every CTA streams about the same number of bytes; the LM head's in contiguous ranges, which make a
+  // CTA's slice of the vocabulary
+  const int n_phase = 4 * h->L + 1;
+  std::vector<std::vector<uint32_t>> units(n_cta);
+  std::vector<uint16_t> pstart((size_t)n_cta * (n_phase + 1));
+  int next = 0;
+  for (int p = 0; p <= n_phase; ++p) {
+    for (int c = 0; c < n_cta; ++c) pstart[(size_t)c * (n_phase + 1) + p] = (uint16_t)units[c].size();
+    if (p == n_phase) break;
+    const int kind = p == n_phase - 1 ? KIND_LM : (p & 3), nt = A.geom[kind].n_tiles;
+    if (kind == KIND_LM) {
+      for (int c = 0; c < n_cta; ++c)
+        for (int t = (int)((long long)c * nt / n_cta); t < (int)((long long)(c + 1) * nt / n_cta); ++t) units[c].push_back(unit_pack(kind, p >> 2, t, 0));
+      continue;
+    }
+    for (int t = 0; t < nt; ++t, next = (next + 1) % n_cta)
+      for (int sub = 0; sub < A.geom[kind].nsub; ++sub) units[next].push_back(unit_pack(kind, p >> 2, t, sub));
+  }
+  A.max_units = 0;
+  for (const auto& u : units) A.max_units = std::max(A.max_units, (int)u.size());
+  if (A.max_units > kMaxUnits) return TABED_OK;
+  std::vector<uint32_t> ulist((size_t)n_cta * A.max_units);
+  for (int c = 0; c < n_cta; ++c) std::copy(units[c].begin(), units[c].end(), ulist.begin() + (size_t)c * A.max_units);
   {
     // wider steps of many rows stay where they were measured
     const int slots = prepass ? h->R : 2 * h->R;
@@ -558,29 +579,6 @@ int setup_persistent(tabed_handle* h) {
     h->allocs.push_back(ptr);
     h->packed = reinterpret_cast<unsigned char*>(ptr);
   }
-  // every CTA's units of a decoder step: the tiles of a phase are dealt round-robin over the CTAs, starting where the phase
-  // before stopped, so that every CTA streams about the same number of bytes; the LM head's in contiguous ranges, which make a
-  // CTA's slice of the vocabulary
-  const int n_phase = 4 * h->L + 1;
-  std::vector<std::vector<uint32_t>> units(n_cta);
-  std::vector<uint16_t> pstart((size_t)n_cta * (n_phase + 1));
-  int next = 0;
-  for (int p = 0; p <= n_phase; ++p) {
-    for (int c = 0; c < n_cta; ++c) pstart[(size_t)c * (n_phase + 1) + p] = (uint16_t)units[c].size();
-    if (p == n_phase) break;
-    const int kind = p == n_phase - 1 ? KIND_LM : (p & 3), nt = A.geom[kind].n_tiles;
-    if (kind == KIND_LM) {
-      for (int c = 0; c < n_cta; ++c)
-        for (int t = (int)((long long)c * nt / n_cta); t < (int)((long long)(c + 1) * nt / n_cta); ++t) units[c].push_back(unit_pack(kind, p >> 2, t, 0));
-      continue;
-    }
-    for (int t = 0; t < nt; ++t, next = (next + 1) % n_cta)
-      for (int sub = 0; sub < A.geom[kind].nsub; ++sub) units[next].push_back(unit_pack(kind, p >> 2, t, sub));
-  }
-  A.max_units = 0;
-  for (const auto& u : units) A.max_units = std::max(A.max_units, (int)u.size());
-  std::vector<uint32_t> ulist((size_t)n_cta * A.max_units);
-  for (int c = 0; c < n_cta; ++c) std::copy(units[c].begin(), units[c].end(), ulist.begin() + (size_t)c * A.max_units);
   uint16_t* d_pstart = nullptr;
   uint32_t* d_ulist = nullptr;
   A2(&d_pstart, pstart.size()); A2(&d_ulist, ulist.size());

@@ -72,6 +72,7 @@ def blank_drafter(cfg):
 @pytest.mark.parametrize("cfg,persistent", [
     (W.DrafterCfg(1, 32, 1, 1, 32, 1 << 20, "bf16"), True),             # 65536 LM-head tiles, all that a unit's number holds
     (W.DrafterCfg(1, 32, 1, 1, 32, (1 << 20) + 1, "bf16"), False),      # one more
+    (W.DrafterCfg(64, 1280, 20, 5, 5504, 32000, "bf16"), True),         # 64 layers: 712 units a CTA (its phases' rounded up: 1038)
 ])
 def test_path_selection_at_the_bounds(cfg, persistent):
     g = blank_drafter(cfg)
