@@ -128,8 +128,8 @@ extern "C" {
                                       projections if it qualifies, else per-operation                    */
 #define TABED_PATH_PER_OP      1   /* one kernel per operation (any drafter, any number of rows)        */
 #define TABED_PATH_PERSISTENT  2   /* the whole round in one cooperative kernel: bf16 drafter, tree_width 1,
-                                      B*m <= 8 rows (with more than 4 rows at least two layers: the first of
-                                      two pending tokens then gets a weight pass of its own), d_model <= 2048
+                                      B*m <= 8 rows (with more than 4 rows the first of two pending tokens
+                                      gets a weight pass of its own), d_model <= 2048
                                       (<= 1024 with more than 4 slots: 3 - 4 or 5 - 8 rows) and
                                       a multiple of 16, vocab <= 2^20,
                                       d_ffn a multiple of 16, H <= 64, (H/Hkv)*head_dim <= 512, <= 64 layers,

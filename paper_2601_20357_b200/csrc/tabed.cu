@@ -468,10 +468,9 @@ int setup_persistent(tabed_handle* h) {
   if (c.dtype != TABED_DTYPE_BF16 || h->D > 1) return TABED_OK;      // (the in-kernel draw proposes one candidate per step)
   const int grp = h->H / h->Hkv;
   // up to kPSlots / 2 rows both pending tokens of a fully accepted block share the first step's weight pass (2 R slots);
-  // with more rows (up to kPSlots) the first of them gets a pass of its own, which needs two layers for its cache
-  // writes to be ordered before the first step's reads
+  // with more rows (up to kPSlots) the first of them gets a pass of its own
   const bool prepass = 2 * h->R > kPSlots;
-  if (h->R > kPSlots || (prepass && h->L < 2) || h->B > kPSlots || h->d % 16 || h->d > kPMaxD || h->F % 16 || (h->Hkv * h->hd) % 16 ||
+  if (h->R > kPSlots || h->B > kPSlots || h->d % 16 || h->d > kPMaxD || h->F % 16 || (h->Hkv * h->hd) % 16 ||
       grp > kMaxGroup || grp * h->hd > 512 || h->L > kPMaxL || h->H > kPMaxHeads || (h->cap + 127) / 128 > kAttnSplitMax)
     return TABED_OK;
   cudaDeviceProp prop;

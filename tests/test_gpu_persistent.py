@@ -125,6 +125,23 @@ def test_lockstep_five_to_eight_rows_mixed_pending(B, m):
     pair.gpu.destroy()
 
 
+@pytest.mark.parametrize("kw", [
+    # one layer: the extra pass is QKV, attention, O and down of that layer alone, and step 0 reads its cache rows
+    dict(layers=1, m=1, B=6, sigma=0.0, prefixes=((("tokens", 95),),), alpha=(1.0,), cid=101, policy=W.POLICY_STATIC),
+], ids=["one_layer"])
+def test_lockstep_branches_that_few_shapes_take(kw):
+    kw = dict(kw)
+    lens = kw.pop("synthetic", None)
+    wl = wl_small(**kw)
+    if lens:
+        wl = wl.replace(synthetic_kv_len=(1, 1))
+    pair = H.build_pair(wl, None if lens is None else np.array(lens))
+    assert pair.gpu.current_path() == TB.PATH_PERSISTENT
+    for rnd in range(3):
+        H.lockstep_round(pair, rnd, override=True)
+    pair.gpu.destroy()
+
+
 @pytest.mark.parametrize("heads,kv_heads,d", [(8, 2, 256), (2, 1, 256), (4, 4, 512)])
 def test_lockstep_head_sizes(heads, kv_heads, d):
     """head_dim 32 (8 heads, 4 per KV head), 128 (2 heads sharing one KV head), 128 without grouping."""
