@@ -129,9 +129,8 @@ extern "C" {
 #define TABED_PATH_PER_OP      1   /* one kernel per operation (any drafter, any number of rows)        */
 #define TABED_PATH_PERSISTENT  2   /* the whole round in one cooperative kernel: bf16 drafter, tree_width 1,
                                       B*m <= 8 rows (with more than 4 rows the first of two pending tokens
-                                      gets a weight pass of its own), d_model <= 2048
-                                      (<= 1024 with more than 4 slots: 3 - 4 or 5 - 8 rows) and
-                                      a multiple of 16, vocab <= 2^20,
+                                      gets a weight pass of its own), d_model <= 2048 (<= 1280 with 3, 4 or
+                                      6 - 8 rows, <= 1536 with 5) and a multiple of 16, vocab <= 2^20,
                                       d_ffn a multiple of 16, H <= 64, (H/Hkv)*head_dim <= 512, <= 64 layers,
                                       kv_capacity <= 32768                                                */
 #define TABED_PATH_TENSOR_CORE 3   /* one kernel per operation with the projections as tcgen05 contractions

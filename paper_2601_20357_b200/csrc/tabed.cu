@@ -519,9 +519,13 @@ int setup_persistent(tabed_handle* h) {
   std::vector<uint32_t> ulist((size_t)n_cta * A.max_units);
   for (int c = 0; c < n_cta; ++c) std::copy(units[c].begin(), units[c].end(), ulist.begin() + (size_t)c * A.max_units);
   {
-    // wider steps of many rows stay where they were measured
+    // Wide steps of many slots are as fast one launch per operation: there the products fill the tensor cores' rows, here a
+    // warp holds 14 - 24 blocks of a row in two batches.  us per pass of two rounds of 3 drafts, 3 / 4 / 6 / 8 rows, 4 layers,
+    // a kernel per operation -> this one: 1088 columns 1263 / 1258 / 1356 / 1379 -> 893 / 927 / 997 / 1084, 1280 columns
+    // 1350 / 1343 / 1448 / 1486 -> 1233 / 1254 / 1301 / 1401, 1536 columns 1464 / 1451 / 1537 / 1573 -> 1423 / 1450 / 1559 / 1663;
+    // up to 4 slots: 1280 columns, 2 rows 1375 -> 1165, 1536 columns, 1 row 1382 -> 1263.
     const int slots = prepass ? h->R : 2 * h->R;
-    if (h->d > 512 * (16 / slots)) return TABED_OK;
+    if (slots > 4 && h->d > (slots > 5 ? 1280 : 1536)) return TABED_OK;
   }
   A.prepass = prepass ? 1 : 0;
   const size_t u_bytes = ((size_t)kPPartFloats + (size_t)kGW * grp * h->hd) * sizeof(float);
