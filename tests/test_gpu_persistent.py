@@ -4,8 +4,8 @@ Same bars as tests/test_gpu_parity.py: with the checker's fp32 logits handed to 
 (lock step), tokens, accept counts, replacement tokens, weights and window sums are bit-exact and
 q, q^(k), p are bitwise equal; the kernel's own forward pass is compared at every step (logits within
 the bf16 bound, probabilities within 1e-5).  The cases here are chosen for what is special in the
-persistent kernel: tiles cut into 1, 2, 4 or 8 sub-units, the ragged last LM-head tile, grouped-query attention with
-head sizes 32/64/128, several attention splits merged by the last CTA to finish, two pending tokens
+persistent kernel: tiles cut into 1 to 8 sub-units, the ragged last LM-head tile, grouped-query attention with
+head sizes 32/64/128, caches in several segments, put together by the CTA with the last one, two pending tokens
 fed in one weight pass (positions produced and consumed in the same phase), greedy mode.
 """
 import numpy as np
@@ -133,7 +133,18 @@ def test_lockstep_five_to_eight_rows_mixed_pending(B, m):
          prefixes=((("tokens", 94),), (("tokens", 33),)), cid=102),
     dict(d=1152, heads=9, kv_heads=3, ffn=1264, vocab=32003, gamma=2, m=2, B=3, sigma=0.02, alpha=(0.9, 0.1),
          prefixes=((("tokens", 40),), (("tokens", 21),)), cid=103),
-], ids=["one_layer", "wide_8_slots", "wide_extra_pass"])
+    # a down tile that takes two rounds of the ring (8 sub-units, rounds of 4), three stages of K and V on their way
+    dict(d=512, heads=8, kv_heads=8, ffn=8192, vocab=32003, gamma=2, cap=4096, synthetic=(4000, 2111, 2592), sigma=0.02,
+         alpha=(0.9, 0.06, 0.04), cid=104),
+    # ... and on a ring of three slots (4 sub-units, rounds of 3)
+    dict(d=1536, heads=24, kv_heads=24, ffn=8960, vocab=64007, gamma=2, m=1, sigma=0.0, alpha=(1.0,), policy=W.POLICY_STATIC,
+         prefixes=((("tokens", 50),),), cid=105),
+    # six rows of a slice of the vocabulary do not fit in shared memory: the exponentials are taken twice
+    dict(d=128, heads=4, kv_heads=2, ffn=272, vocab=152003, gamma=2, m=3, B=2, sigma=0.02, alpha=(0.9, 0.06, 0.04),
+         prefixes=((("tokens", 30),), (("tokens", 60),), (("tokens", 5),)), cid=106),
+    dict(d=128, heads=4, kv_heads=2, ffn=272, vocab=152003, gamma=2, m=3, B=2, sigma=0.02, alpha=(0.9, 0.06, 0.04),
+         prefixes=((("tokens", 30),), (("tokens", 60),), (("tokens", 5),)), cid=107, mode=W.MODE_GREEDY),
+], ids=["one_layer", "wide_8_slots", "wide_extra_pass", "down_two_rounds", "ring_of_three", "slice_beyond_shared_memory", "the_same_greedy"])
 def test_lockstep_branches_that_few_shapes_take(kw):
     """(Probabilities: the checker's own perturbed runs, as below, are at most 3.5e-6 apart at 1280 columns, 2.9e-6 at 1536, 9e-7 at
     512 and 2e-8 with 152003 tokens.)"""
