@@ -993,7 +993,7 @@ __global__ void __launch_bounds__(kPT, 1) k_draft_round(const RoundArgs A) {
           if (++stage == A.kv_stages) stage = 0;
           if (lim > 0) {
             // ---- softmax and P V for all heads of the group at once ----
-            float pw[4];
+            float pw[4], f[2];
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
               // (the maximum is of the rounded products, any reference will do; the weight's exponent is rounded once, behind the
@@ -1002,17 +1002,17 @@ __global__ void __launch_bounds__(kPT, 1) k_draft_round(const RoundArgs A) {
               float mx = fmaxf(x0 * scale2, x1 * scale2);
 #pragma unroll
               for (int o = 4; o < 32; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(FULL, mx, o));
-              const float Mn = fmaxf(m_run[e], mx), N = Mn > -INFINITY ? Mn : 0.0f, f = ex2_approx(m_run[e] - N);
+              const float Mn = fmaxf(m_run[e], mx), N = Mn > -INFINITY ? Mn : 0.0f;
+              f[e] = ex2_approx(m_run[e] - N);
               m_run[e] = Mn;
               pw[e] = ex2_approx(fmaf(x0, scale2, -N)); pw[e + 2] = ex2_approx(fmaf(x1, scale2, -N));
-              l_run[e] = fmaf(l_run[e], f, pw[e] + pw[e + 2]);
-#pragma unroll
-              for (int j = 0; j < MT; ++j) { oc[j][e] *= f; oc[j][e + 2] *= f; }
+              l_run[e] = fmaf(l_run[e], f[e], pw[e] + pw[e + 2]);
             }
             // The weights as bf16 terms of 8 bits (fp32 sums), moved from accumulator layout (positions as rows) to B-operand
             // layout (positions as the summed index): three terms, all of an fp32 weight - two for the cached positions of head size 64.
             // (With two for all of them a sum of 300 positions that cancel is eleven times as far off, at head sizes 32 and 128; the
-            // third costs 2 - 3 % of a round over 6000 positions there, and at head size 64, for the new positions, 1 % at 8192.)
+            // third term costs at most 1 % of a round: 3 rows of 6000 positions at 32 / 128 919 / 1010 -> 907 / 1018 us with
+            // all that is here, of 8192 at 64, where the new positions have it, 4057 -> 4095.)
             uint32_t t0, t1, w0[2], w1[2], w2[2];
             auto term = [&](uint32_t (&w)[2]) {
               t0 = pack_bf16(pw[0], pw[1]); t1 = pack_bf16(pw[2], pw[3]);
@@ -1032,9 +1032,14 @@ __global__ void __launch_bounds__(kPT, 1) k_draft_round(const RoundArgs A) {
             for (int j = 0; j < MT; ++j) {
               uint32_t af[4];
               values(j, af);
-              mma_bf16(oc[j], af, w0);
-              mma_bf16(oc[j], af, w1);
-              if constexpr (HD != 64) mma_bf16(oc[j], af, w2);
+              // (the tensor core's sums are cut off, not rounded: the smallest terms first, and only these 16 positions'.  Sums
+              // carried through it were 9 % further off at head size 32; 8192 positions 4098 -> 4139 us)
+              float t[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+              if constexpr (HD != 64) mma_bf16(t, af, w2);
+              mma_bf16(t, af, w1);
+              mma_bf16(t, af, w0);
+#pragma unroll
+              for (int e = 0; e < 4; ++e) oc[j][e] = fmaf(oc[j][e], f[e & 1], t[e]);
             }
             if (HD == 64 && cached < 16) {
               remainder(); term(w2);
