@@ -520,14 +520,18 @@ __device__ __noinline__ Found find_mass(const uint2* w, int n, bool draw, float 
 // ------------------------------------------------------------------------------------------------
 // the kernel
 // ------------------------------------------------------------------------------------------------
-// HD: head size.  NF: blocks of 16 input columns that a warp holds of a row (a group's warps share the row's blocks).
+// HD: head size.  NF: blocks of 16 input columns that a warp holds of a row (a group's warps share the row's blocks); the code
+// is that long in every phase that normalises, so a row takes the shortest that holds it (NF 6 against 8, us per pass of three
+// rounds, 1 / 3 / 6 rows: 256 columns 723 / 781 / 900 against 748 / 796 / 918, 576 columns 819 / 897 / 1139 against 839 / 910 / 1160).
 //
 // What bounds a phase is the chain from the arrival of its words to the departure of its results, and on that chain the number
 // of instructions that the CTA's warps issue (16 warps that all run 500 instructions take 2000 cycles of the four
 // schedulers, twice that out of the instruction cache's next level).  Hence two groups of six warps that take turns: group 0
 // has the phases that normalise (QKV, gate/up, LM head), group 1 the others (attention, O, down).  While a group works, the
-// other one has already set up its next phase and polls for its words.  Twelve warps have 168 registers a thread, with
-// which no phase spills on its way.
+// other one has already set up its next phase and polls for its words.  Twelve warps have 168 registers a thread.
+// With those nothing is spilled at head size 64 up to NF 8 and at 32 up to NF 12; elsewhere bytes of spill stores a thread: head
+// size 64 28 / 412 at NF 12 / 24, 32 292 at NF 24, 128 128 - 164 up to NF 12 and 540 at 24 (with TRACE more, up to 1284: a
+// timeline's phases are that much longer than an untraced round's).
 template <int HD, int NF, bool TRACE>
 __global__ void __launch_bounds__(kPT, 1) k_draft_round(const RoundArgs A) {
   extern __shared__ __align__(128) unsigned char dyn_smem[];

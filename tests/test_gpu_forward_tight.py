@@ -159,7 +159,7 @@ def test_attention_weights_carry_fp32(hd):
     for name in ("wv", "w_down"):
         weights[name][0] = np.zeros_like(weights[name][0])
     weights["lm_head"] = np.eye(d, dtype=np.float32)
-    # the weights of the cached positions, from the checker's own q (the first step appends position n)
+    # the weights of the cached positions, from the oracle's own q (the first step appends position n)
     probe = OracleDrafter(cfg, weights)
     a = probe.rb(probe.rmsnorm(x[None].astype(np.float64), probe.layers[0]["norm1"]))
     rotated = lambda w: probe.rb(probe.rope((a @ w.T).reshape(1, heads, hd), np.array([n])))[0]

@@ -146,7 +146,7 @@ def test_lockstep_five_to_eight_rows_mixed_pending(B, m):
          prefixes=((("tokens", 30),), (("tokens", 60),), (("tokens", 5),)), cid=107, mode=W.MODE_GREEDY),
 ], ids=["one_layer", "wide_8_slots", "wide_extra_pass", "down_two_rounds", "ring_of_three", "slice_beyond_shared_memory", "the_same_greedy"])
 def test_lockstep_branches_that_few_shapes_take(kw):
-    """(Probabilities: the checker's own perturbed runs, as below, are at most 3.5e-6 apart at 1280 columns, 2.9e-6 at 1536, 9e-7 at
+    """(Probabilities: the oracle's own perturbed runs, as below, are at most 3.5e-6 apart at 1280 columns, 2.9e-6 at 1536, 9e-7 at
     512 and 2e-8 with 152003 tokens.)"""
     kw = dict(kw)
     lens = kw.pop("synthetic", None)
@@ -186,7 +186,7 @@ def test_lockstep_ragged_vocabulary_and_greedy():
 def test_lockstep_edges_of_chunks_blocks_and_slices(d, heads, kv_heads, ffn, vocab, lens):
     """Shapes at which a warp's share of the columns, a CTA's slice of the vocabulary or a chunk of a cache is ragged, empty or
     exactly full; small noise, so that some blocks are fully accepted and two positions are produced in one phase (on both sides
-    of a chunk's end).  Vocabularies are large enough for the bar of 1e-5 on probabilities: two runs of the checker that differ by
+    of a chunk's end).  Vocabularies are large enough for the bar of 1e-5 on probabilities: two runs of the oracle that differ by
     1e-7 before every rounding (test_oracle_drafter.py's perturbation; three steps behind these prefixes, four seeds a row) are at
     most 3.5e-6 apart at 1280 columns, 2.2e-6 at 1152, 2.8e-6 at 640, 3.4e-6 at 576 and 2.6e-6 below.  (With 8009 tokens it was
     1.15e-5 and 5.7e-6 at 1280 and 1152, where the likeliest token has p = 2.4e-3: rounding alone was on the bar.)"""
